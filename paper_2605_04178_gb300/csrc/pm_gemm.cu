@@ -23,8 +23,6 @@
 // tile i+1 starts on row block 0 while the epilogue still drains row block 1.  Each CTA of a pair loads its own A
 // rows and half of B (traffic 2 M_A + M_B per pair, no multicast); the pair
 // leader issues the cta_group::2 MMAs.
-#include <cuda_bf16.h>
-#include <cuda_fp8.h>
 #include <stdlib.h>
 
 #include <algorithm>
@@ -536,88 +534,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   }
 }
 
-// --------------------------------------------------------------- operand prep
-// Row-major FP32 inputs to the tensor-core operand formats.  HBM-bound
-// pre-passes outside the GEMM proper.
-__device__ __forceinline__ float tf32_rn(float x) {
-  // round to nearest even at mantissa bit 13 (finite inputs)
-  uint32_t b = __float_as_uint(x);
-  if ((b & 0x7f800000u) == 0x7f800000u) return x;
-  b = (b + 0xfffu + ((b >> 13) & 1u)) & 0xffffe000u;
-  return __uint_as_float(b);
-}
-
-__global__ void amax_kernel(const float* __restrict__ x, int64_t n, unsigned int* __restrict__ amax_bits) {
-  float m = 0.f;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    m = fmaxf(m, fabsf(__ldg(x + i)));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(amax_bits, __float_as_uint(m));
-}
-
-__device__ __forceinline__ float fp8_scale_of(unsigned int amax_bits) {
-  const float amax = __uint_as_float(amax_bits);
-  return amax > 0.f ? 448.f / amax : 1.f;
-}
-
-// Row-major [R, C] FP32 -> same layout in the operand format (A side).
-__global__ void convert_rows_kernel(const float* __restrict__ x, int64_t n, int mode, void* __restrict__ y,
-                                    float* __restrict__ y_lo, const unsigned int* __restrict__ amax_bits,
-                                    float* __restrict__ scale_out) {
-  float s = 1.f;
-  if (mode == PM_FP8E4M3) {
-    s = fp8_scale_of(*amax_bits);
-    if (blockIdx.x == 0 && threadIdx.x == 0 && scale_out) *scale_out = s;
-  }
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const float v = __ldg(x + i);
-    if (mode == PM_BF16) {
-      static_cast<__nv_bfloat16*>(y)[i] = __float2bfloat16_rn(v);
-    } else if (mode == PM_FP8E4M3) {
-      static_cast<__nv_fp8_storage_t*>(y)[i] = __nv_cvt_float_to_fp8(v * s, __NV_SATFINITE, __NV_E4M3);
-    } else {
-      const float hi = tf32_rn(v);
-      static_cast<float*>(y)[i] = hi;
-      y_lo[i] = tf32_rn(v - hi);
-    }
-  }
-}
-
-// Row-major [K, N] FP32 -> K-major [N, K] operand (B side), 32x32 tiles.
-__global__ void transpose_convert_kernel(const float* __restrict__ x, int K, int N, int mode, void* __restrict__ y,
-                                         float* __restrict__ y_lo, const unsigned int* __restrict__ amax_bits,
-                                         float* __restrict__ scale_out) {
-  __shared__ float tile[32][33];
-  float s = 1.f;
-  if (mode == PM_FP8E4M3) {
-    s = fp8_scale_of(*amax_bits);
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0 && scale_out) *scale_out = s;
-  }
-  const int n0 = blockIdx.x * 32, k0 = blockIdx.y * 32;
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const int k = k0 + r, nn = n0 + threadIdx.x;
-    tile[r][threadIdx.x] = (k < K && nn < N) ? __ldg(x + (size_t)k * N + nn) : 0.f;
-  }
-  __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const int nn = n0 + r, k = k0 + threadIdx.x;
-    if (nn < N && k < K) {
-      const float v = tile[threadIdx.x][r];
-      const size_t o = (size_t)nn * K + k;
-      if (mode == PM_BF16) {
-        static_cast<__nv_bfloat16*>(y)[o] = __float2bfloat16_rn(v);
-      } else if (mode == PM_FP8E4M3) {
-        static_cast<__nv_fp8_storage_t*>(y)[o] = __nv_cvt_float_to_fp8(v * s, __NV_SATFINITE, __NV_E4M3);
-      } else {
-        const float hi = tf32_rn(v);
-        static_cast<float*>(y)[o] = hi;
-        y_lo[o] = tf32_rn(v - hi);
-      }
-    }
-  }
-}
-
 // ------------------------------------------------------------------ host side
 static inline int dt_elem(int dt) { return dt == PM_FP32 ? 4 : (dt == PM_BF16 ? 2 : 1); }
 static inline int dt_halves(int dt) { return dt == PM_FP32 ? 2 : 1; }
@@ -911,37 +827,6 @@ extern "C" pm_status pm_gemm_operand_bytes(int32_t dtype, int32_t M, int32_t N, 
   return PM_OK;
 }
 
-extern "C" pm_status pm_gemm_prepare(int32_t dtype, const float* A_dev, const float* B_dev, int32_t M, int32_t N,
-                                     int32_t K, void* A_op_dev, void* B_op_dev, float* scales_dev, void* stream) {
-  PM_REQUIRE(dtype >= 0 && dtype <= 2 && M > 0 && N > 0 && K > 0, PM_EINVAL, "bad dtype or shape");
-  PM_REQUIRE(A_dev && B_dev && A_op_dev && B_op_dev, PM_EINVAL, "null pointer");
-  PM_REQUIRE(dtype != PM_FP8E4M3 || scales_dev, PM_EINVAL, "FP8 needs scales_dev (4 floats)");
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const int sms = std::max(1, sm_count());
-  const int64_t nA = (int64_t)M * K, nB = (int64_t)K * N;
-  unsigned int* amax = nullptr;
-  if (dtype == PM_FP8E4M3) {
-    amax = reinterpret_cast<unsigned int*>(scales_dev + 2);
-    PM_CUDA(cudaMemsetAsync(amax, 0, 2 * sizeof(unsigned int), s));
-    amax_kernel<<<sms * 4, 256, 0, s>>>(A_dev, nA, amax);
-    amax_kernel<<<sms * 4, 256, 0, s>>>(B_dev, nB, amax + 1);
-    pm_status st = launch_status("amax_kernel");
-    if (st != PM_OK) return st;
-  }
-  float* a_lo = dtype == PM_FP32 ? static_cast<float*>(A_op_dev) + nA : nullptr;
-  float* b_lo = dtype == PM_FP32 ? static_cast<float*>(B_op_dev) + (int64_t)N * K : nullptr;
-  convert_rows_kernel<<<sms * 8, 256, 0, s>>>(A_dev, nA, dtype, A_op_dev, a_lo, amax,
-                                              dtype == PM_FP8E4M3 ? scales_dev : nullptr);
-  pm_status st = launch_status("convert_rows_kernel");
-  if (st != PM_OK) return st;
-  dim3 grid((N + 31) / 32, (K + 31) / 32);
-  PM_REQUIRE(grid.y <= 65535, PM_EINVAL, "K too large for the transpose grid");
-  transpose_convert_kernel<<<grid, dim3(32, 8), 0, s>>>(B_dev, K, N, dtype, B_op_dev, b_lo,
-                                                          amax ? amax + 1 : nullptr,
-                                                          dtype == PM_FP8E4M3 ? scales_dev + 1 : nullptr);
-  return launch_status("transpose_convert_kernel");
-}
-
 extern "C" pm_status pm_gemm_run(const pm_cfg* cfg, const void* A_op_dev, const void* B_op_dev, float* C_dev,
                                  const float* scales_dev, void* stream) {
   PM_REQUIRE(cfg != nullptr, PM_EINVAL, "cfg is NULL");
@@ -1170,8 +1055,7 @@ extern "C" pm_status pm_gemm_host(const pm_cfg* cfg, const float* A_host, const 
   float* b32 = reinterpret_cast<float*>(ws + Lh.off_b32);
   void* bop = ws + Lh.off_bop;
   float* scales = reinterpret_cast<float*>(ws + Lh.off_scales);
-  unsigned int* amax = reinterpret_cast<unsigned int*>(scales + 2);
-  const int sms = std::max(1, sm_count());
+  PM_REQUIRE((K + 31) / 32 <= 65535, PM_EINVAL, "K too large for the transpose grid");
   PM_CUDA(cudaEventRecord(P.start, caller));
   PM_CUDA(cudaStreamWaitEvent(P.s_in, P.start, 0));
   PM_CUDA(cudaStreamWaitEvent(P.s_comp, P.start, 0));
@@ -1180,16 +1064,8 @@ extern "C" pm_status pm_gemm_host(const pm_cfg* cfg, const float* A_host, const 
   PM_CUDA(cudaMemcpyAsync(b32, B_host, (size_t)K * N * 4, cudaMemcpyHostToDevice, P.s_in));
   PM_CUDA(cudaEventRecord(P.b_ready, P.s_in));
   PM_CUDA(cudaStreamWaitEvent(P.s_comp, P.b_ready, 0));
-  if (dt == PM_FP8E4M3) {
-    PM_CUDA(cudaMemsetAsync(amax, 0, 2 * sizeof(unsigned int), P.s_comp));
-    amax_kernel<<<sms * 4, 256, 0, P.s_comp>>>(b32, (int64_t)K * N, amax + 1);
-  }
-  dim3 tgrid((N + 31) / 32, (K + 31) / 32);
-  PM_REQUIRE(tgrid.y <= 65535, PM_EINVAL, "K too large for the transpose grid");
-  transpose_convert_kernel<<<tgrid, dim3(32, 8), 0, P.s_comp>>>(
-      b32, K, N, dt, bop, dt == PM_FP32 ? static_cast<float*>(bop) + (int64_t)N * K : nullptr,
-      dt == PM_FP8E4M3 ? amax + 1 : nullptr, dt == PM_FP8E4M3 ? scales + 1 : nullptr);
-  st = launch_status("transpose_convert_kernel");
+  if (dt == PM_FP8E4M3) PM_CUDA(cudaMemsetAsync(scales + 2, 0, 2 * sizeof(unsigned int), P.s_comp));
+  st = launch_prepare(dt, nullptr, 0, b32, K, N, nullptr, bop, scales, P.s_comp);
   if (st != PM_OK) return st;
   // A in row chunks
   const int nch = (int)((M + Lh.Mc - 1) / Lh.Mc);
@@ -1204,13 +1080,7 @@ extern "C" pm_status pm_gemm_host(const pm_cfg* cfg, const float* A_host, const 
     PM_CUDA(cudaMemcpyAsync(a32, A_host + r0 * K, (size_t)rows * K * 4, cudaMemcpyHostToDevice, P.s_in));
     PM_CUDA(cudaEventRecord(P.a_loaded[j], P.s_in));
     PM_CUDA(cudaStreamWaitEvent(P.s_comp, P.a_loaded[j], 0));
-    const int64_t nA = (int64_t)rows * K;
-    if (dt == PM_FP8E4M3) amax_kernel<<<sms * 4, 256, 0, P.s_comp>>>(a32, nA, amax);
-    convert_rows_kernel<<<sms * 8, 256, 0, P.s_comp>>>(a32, nA, dt, aop,
-                                                       dt == PM_FP32 ? static_cast<float*>(aop) + nA : nullptr,
-                                                       dt == PM_FP8E4M3 ? amax : nullptr,
-                                                       dt == PM_FP8E4M3 ? scales : nullptr);
-    st = launch_status("convert_rows_kernel");
+    st = launch_prepare(dt, a32, rows, nullptr, K, N, aop, nullptr, scales, P.s_comp);
     if (st != PM_OK) return st;
     PM_CUDA(cudaEventRecord(P.a_free[j], P.s_comp));
     if (i >= 2) PM_CUDA(cudaStreamWaitEvent(P.s_comp, P.c_free[j], 0));

@@ -24,6 +24,9 @@ unsigned int* watchdog_word();
 unsigned long long watchdog_limit_ns();
 // Number of SMs of the current device.
 int sm_count();
+// Operand preparation on stream s (pm_prepare.cu): A (rows x K, nullptr: none) and B (K x N, nullptr: none).
+pm_status launch_prepare(int dt, const float* A, int64_t rows, const float* B, int K, int N, void* A_op, void* B_op,
+                         float* scales, cudaStream_t s);
 // Resources pm_shutdown releases: the library's stream pool (all devices), and
 // the calling thread's host-transfer pipeline and tensor-map caches.
 void release_stream_pool();
