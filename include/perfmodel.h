@@ -7,7 +7,8 @@
  *  - Pointers named *_dev are CUDA device pointers on the current device; the
  *    caller allocates and owns them.  Pointers named *_host are host memory.
  *    The library keeps only a small per-device cache (TMA descriptors of the
- *    last call, the watchdog word) and never frees caller memory.
+ *    last call, the watchdog word), a page-locked host block per thread for the
+ *    grouped model calls, and never frees caller memory.
  *  - `stream` is a cudaStream_t passed as void* (NULL = legacy default
  *    stream).  Entry points documented "async" only enqueue work; those
  *    documented "synchronises" wait for their stream before returning.
@@ -376,8 +377,9 @@ pm_status pm_autotune_pick(const int32_t* MNK_dev, int64_t n, int32_t dtype, con
  * order reversed on odd rounds when G > 1; T_hat = launch + max_w sum of the
  * worker's tau, launch = T_launch, plus L_alloc + L_dealloc under the
  * measured reading).  Host arrays of G entries (G <= 1024); *t_pred_host in
- * seconds, NaN for a cta_group 2 launch when n_sm < 2.  Allocates a few KB
- * of stream-ordered device scratch.  Synchronises. */
+ * seconds, NaN for a cta_group 2 launch when n_sm < 2.  The grouped model calls
+ * keep one 87 KB block of page-locked host memory per calling thread, until the
+ * thread ends or calls pm_shutdown.  Synchronises. */
 pm_status pm_grouped_predict(int32_t G, const int32_t* M_host, int32_t N, int32_t K, const int16_t* BM_host,
                              const int16_t* BN_host, int32_t BK, int32_t stages, int32_t cta_group, int32_t dtype,
                              const pm_params* theta_host, int32_t n_sm, float* t_pred_host, void* stream);
@@ -478,7 +480,8 @@ const char* pm_last_error(void);
 
 /* Releases what the library holds beyond its static device arrays: its pool
  * of concurrent-probe streams on every device, and the calling thread's
- * host-transfer pipeline (streams, events) and TMA descriptor caches; it also
+ * host-transfer pipeline (streams, events), page-locked block of the grouped
+ * model calls and TMA descriptor caches; it also
  * forgets the cached device addresses of the static arrays (the watchdog
  * word, the allocation-free gradient's scratch) and the cached SM counts.
  * Call it before a device reset (cudaDeviceReset reloads the module, so a

@@ -729,22 +729,37 @@ __global__ void __launch_bounds__(kTuneThreads) autotune_topk_kernel(const int32
 // with that group's (BM, BN) and the launch's (BK, stages, cta_group), and
 // the launch ends with its busiest worker:
 //   T_hat = launch + max_w sum_q n_{w,q} tau_q.
-constexpr int kGroupThreads = 256;
+constexpr int kGroupThreads = 256;       // one launch's makespan and its gradient
+constexpr int kGroupTuneThreads = 1024;  // the tuner: a thread per (group, tile)
 constexpr int kMaxGroups = 1024;
+constexpr int kGroupClasses = 6;         // tile areas 4096 << 4 .. 4096 << 0, then none
 
-__device__ __forceinline__ int64_t count_congruent(int64_t X, int64_t w, int64_t n) {
-  // number of t in [0, X] with t = w (mod n), for X >= -1
-  return X < w ? 0 : (X - w) / n + 1;
-}
+// The launch's schedule.  list[i] = the group at position i of the launch's
+// list (pos[q] the position of group q), tau[i] = its tile time, and the first
+// position past it,
+// off[i + 1] = sum of the listed groups' tiles, kept as off = per * P + rem with
+// P the period of the deal (n workers dealt plainly, 2 n when odd rounds are
+// reversed): a worker's share of any range of positions is then two compares
+// (dealt_before) instead of 64-bit divisions per worker and group.
+template <class F>
+struct Schedule {
+  F tau[kMaxGroups];
+  int64_t per[kMaxGroups + 1];
+  int rem[kMaxGroups + 1];
+  int16_t list[kMaxGroups], pos[kMaxGroups];
+  uint8_t key[kMaxGroups];               // class << 5 | rank inside its 32 groups
+  int cls[kGroupClasses][32];            // groups per class and 32 groups, then their first positions
+  int cls_total[kGroupClasses];
+  int64_t part[32];                      // tiles per 32 positions, then their first position
+};
 
-// How many of the listed positions [a, b) are dealt to worker w of n.
-// Reversing odd rounds gives position i to worker w exactly when
-// i mod 2n is w or 2n - 1 - w.
-__device__ __forceinline__ int64_t dealt(int64_t a, int64_t b, int64_t w, int64_t n, bool reverse_odd) {
-  if (!reverse_odd) return count_congruent(b - 1, w, n) - count_congruent(a - 1, w, n);
-  const int64_t p = 2 * n, w2 = p - 1 - w;
-  return count_congruent(b - 1, w, p) - count_congruent(a - 1, w, p) + count_congruent(b - 1, w2, p) -
-         count_congruent(a - 1, w2, p);
+// How many of the positions [0, off[i]) are dealt to worker w: position t goes
+// to worker t mod n, or with reversed odd rounds to the w with t mod 2n in
+// {w, 2n - 1 - w}.
+template <class F>
+__device__ __forceinline__ int64_t dealt_before(const Schedule<F>& sc, int i, int64_t w, int64_t n, bool rev) {
+  const int64_t r = sc.rem[i];
+  return rev ? 2 * sc.per[i] + (r > w) + (r > 2 * n - 1 - w) : sc.per[i] + (r > w);
 }
 
 // Working set of a grouped launch (every group's A rows, its B and its C),
@@ -756,31 +771,82 @@ __device__ F grouped_working_set(const int32_t* Mg, int G, int N, int K, int dt)
   __syncthreads();
   unsigned long long mine = 0ull;
   for (int q = threadIdx.x; q < G; q += blockDim.x) mine += (unsigned long long)Mg[q];
-  atomicAdd(&sum_m, mine);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+  if ((threadIdx.x & 31) == 0) atomicAdd(&sum_m, mine);
   __syncthreads();
   const F sm = (F)sum_m;
-  __syncthreads();
   return (F)dt_loads(dt) * (F)dt_bytes(dt) * (sm * (F)K + (F)G * (F)N * (F)K) + F(4) * sm * (F)N;
 }
 
-// The launch's list of groups: list[i] = the group at position i, off[i] =
-// its first tile; tiles[q] = group q's tiles.  Largest tile area first
-// (area / 4096 = 2^class, class 0..4; a group without a valid tile, area 0,
-// last), ties in the caller's order.  Called by all threads.
-__device__ void grouped_list(const int16_t* bm, const int16_t* bn, const int64_t* tiles, int G, int16_t* list,
-                             int64_t* off) {
-  if (threadIdx.x == 0) {
-    int k = 0;
-    if (G > 1) {
-      for (int cls = 4; cls >= -1; --cls)
-        for (int q = 0; q < G; ++q)
-          if (__ffs(((int)bm[q] * (int)bn[q]) >> 12) - 1 == cls) list[k++] = (int16_t)q;
-    } else {
-      list[0] = 0;
-    }
-    off[0] = 0;
-    for (int i = 0; i < G; ++i) off[i + 1] = off[i] + tiles[list[i]];
+// Inclusive sum over the warp's lanes.
+__device__ __forceinline__ int64_t warp_scan(int64_t v) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t u = __shfl_up_sync(0xffffffffu, v, o);
+    if ((int)(threadIdx.x & 31) >= o) v += u;
   }
+  return v;
+}
+
+// Lists the launch's groups: largest tile area first (area / 4096 = 2^class,
+// class 4..0; a group without a valid tile, area 0, last), ties in the caller's
+// order: a counting sort over 32-group pieces with warp votes, then a prefix
+// sum of the listed tiles.  tiles[q] by group; sc.tau is the caller's to fill.
+// Called by all threads (blockDim a multiple of 32, at least six warps).
+template <class F>
+__device__ void grouped_list(const int16_t* bm, const int16_t* bn, const int64_t* tiles, int G, int64_t n_conc,
+                             Schedule<F>& sc) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+  const int pieces = (G + 31) >> 5;
+  for (int pc = warp; pc < pieces; pc += n_warps) {
+    const int q = 32 * pc + lane;
+    // 0: area 16 * 4096 .. 4: 4096, 5: no tile (G = 1 is its own order)
+    const int c = q < G ? 5 - __ffs(((int)bm[q] * (int)bn[q]) >> 12) : -1;
+#pragma unroll
+    for (int k = 0; k < kGroupClasses; ++k) {
+      const unsigned m = __ballot_sync(0xffffffffu, c == k);
+      if (c == k) sc.key[q] = (uint8_t)((k << 5) | __popc(m & ((1u << lane) - 1u)));
+      if (lane == 0) sc.cls[k][pc] = __popc(m);
+    }
+  }
+  __syncthreads();
+  if (warp < kGroupClasses) {
+    const int v = lane < pieces ? sc.cls[warp][lane] : 0;
+    const int inc = (int)warp_scan(v);
+    if (lane < pieces) sc.cls[warp][lane] = inc - v;
+    if (lane == 31) sc.cls_total[warp] = inc;
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < G; q += blockDim.x) {
+    const int key = sc.key[q], c = key >> 5;
+    int i = sc.cls[c][q >> 5] + (key & 31);
+    for (int k = 0; k < c; ++k) i += sc.cls_total[k];
+    sc.list[i] = (int16_t)q;
+    sc.pos[q] = (int16_t)i;
+  }
+  __syncthreads();
+  for (int pc = warp; pc < pieces; pc += n_warps) {
+    const int i = 32 * pc + lane;
+    const int64_t inc = warp_scan(i < G ? tiles[sc.list[i]] : 0);
+    if (i < G) sc.per[i + 1] = inc;
+    if (lane == 31) sc.part[pc] = inc;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const int64_t v = lane < pieces ? sc.part[lane] : 0;
+    const int64_t inc = warp_scan(v);
+    if (lane < pieces) sc.part[lane] = inc - v;
+  }
+  __syncthreads();
+  const int64_t P = G > 1 ? 2 * n_conc : n_conc;
+  for (int i = threadIdx.x; i < G; i += blockDim.x) {
+    const int64_t off = sc.per[i + 1] + sc.part[i >> 5];
+    const int64_t per = P > 0 ? off / P : 0;      // no worker: the caller rejects the launch
+    sc.per[i + 1] = per;
+    sc.rem[i + 1] = (int)(off - per * P);
+  }
+  if (threadIdx.x == 0) { sc.per[0] = 0; sc.rem[0] = 0; }
   __syncthreads();
 }
 
@@ -788,36 +854,41 @@ __device__ void grouped_list(const int16_t* bm, const int16_t* bn, const int64_t
 // busy_w adds n_{w,q} tau_q over the list in order.  Called by all threads;
 // the result is valid in every thread.
 template <class F>
-__device__ F grouped_makespan(const F* tau, const int16_t* list, const int64_t* off, int G, int64_t n_conc,
-                              int* w_star) {
-  __shared__ F red_v[kGroupThreads / 32];
-  __shared__ int red_i[kGroupThreads / 32];
+__device__ F grouped_makespan(const Schedule<F>& sc, int G, int64_t n_conc, int* w_star) {
+  __shared__ F red_v[32];
+  __shared__ int red_i[32];
   const bool rev = G > 1;
   F mx = F(-1);
   int mi = 0x7fffffff;
   for (int64_t w = threadIdx.x; w < n_conc; w += blockDim.x) {
     F busy = F(0);
+    int64_t before = 0;
+#pragma unroll 4
     for (int i = 0; i < G; ++i) {
-      const int64_t cnt = dealt(off[i], off[i + 1], w, n_conc, rev);
-      if (cnt) busy += (F)cnt * tau[list[i]];
+      const int64_t upto = dealt_before(sc, i + 1, w, n_conc, rev);
+      const int64_t cnt = upto - before;
+      before = upto;
+      if (cnt) busy += count_to<F>(cnt) * sc.tau[i];
     }
     if (busy > mx) { mx = busy; mi = (int)w; }
   }
+  auto reduce = [&]() {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const F ov = __shfl_xor_sync(0xffffffffu, mx, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, mi, o);
-    if (ov > mx || (ov == mx && oi < mi)) { mx = ov; mi = oi; }
-  }
-  if ((threadIdx.x & 31) == 0) { red_v[threadIdx.x >> 5] = mx; red_i[threadIdx.x >> 5] = mi; }
+    for (int o = 16; o > 0; o >>= 1) {
+      const F ov = __shfl_xor_sync(0xffffffffu, mx, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, mi, o);
+      if (ov > mx || (ov == mx && oi < mi)) { mx = ov; mi = oi; }
+    }
+  };
+  reduce();
+  const int lane = threadIdx.x & 31;
+  if (lane == 0) { red_v[threadIdx.x >> 5] = mx; red_i[threadIdx.x >> 5] = mi; }
   __syncthreads();
-  F m = red_v[0];
-  int i0 = red_i[0];
-  for (int w = 1; w < (int)(blockDim.x / 32); ++w)
-    if (red_v[w] > m || (red_v[w] == m && red_i[w] < i0)) { m = red_v[w]; i0 = red_i[w]; }
-  __syncthreads();
-  if (w_star) *w_star = i0;
-  return m;
+  mx = lane < (int)(blockDim.x >> 5) ? red_v[lane] : F(-1);
+  mi = lane < (int)(blockDim.x >> 5) ? red_i[lane] : 0x7fffffff;
+  reduce();
+  if (w_star) *w_star = mi;
+  return mx;
 }
 
 template <class F>
@@ -832,52 +903,76 @@ __device__ __forceinline__ F launch_time(const ThetaT<F>& th) {
 }
 
 // Grouped autotuner: block b handles launch-level combination b =
-// (BK index, stages, cta_group) in lexicographic order; threads pick each
-// group's (BM, BN) minimising tiles x tau, then the makespan of the launch's
-// schedule is evaluated.
-__global__ void __launch_bounds__(kGroupThreads) grouped_tune_kernel(const int32_t* __restrict__ Mg, int G, int N,
-                                                                     int K, int dt, Theta th, int n_sm,
-                                                                     float* __restrict__ out_t,
-                                                                     int16_t* __restrict__ out_bm,
-                                                                     int16_t* __restrict__ out_bn) {
+// (BK index, stages, cta_group) in lexicographic order; a thread per (group,
+// tile) evaluates the model, a thread per group picks the (BM, BN) minimising
+// tiles x tau, then the makespan of the launch's schedule is evaluated.  The
+// row counts and the results are in the caller's page-locked host memory.
+//
+// Bound: latency (20 blocks, one wave).  Nine threads per group in place of
+// nine evaluations per thread, the counting sort and prefix sum in place of one
+// thread's loops, and no division in the worker loop took the kernel from
+// 84 to 10.7 us at 64 groups.
+__global__ void __launch_bounds__(kGroupTuneThreads) grouped_tune_kernel(const int32_t* __restrict__ Mg, int G, int N,
+                                                                         int K, int dt, Theta th, int n_sm,
+                                                                         float* __restrict__ out_t,
+                                                                         int16_t* __restrict__ out_bm,
+                                                                         int16_t* __restrict__ out_bn) {
+  __shared__ Schedule<float> sc;
+  __shared__ int32_t Ms[kMaxGroups];
   __shared__ float tau[kMaxGroups];
   __shared__ int64_t tiles[kMaxGroups];
-  __shared__ int64_t off[kMaxGroups + 1];
-  __shared__ int16_t bm_s[kMaxGroups], bn_s[kMaxGroups], list[kMaxGroups];
+  __shared__ int16_t bm_s[kMaxGroups], bn_s[kMaxGroups];
+  // the candidates of a pass, in memory that the schedule takes later
+  static_assert(sizeof(sc.per) >= 4 * kGroupTuneThreads && sizeof(sc.rem) >= 4 * kGroupTuneThreads, "candidates");
+  float* const cand_cost = reinterpret_cast<float*>(sc.per);
+  float* const cand_tau = reinterpret_cast<float*>(sc.rem);
   const int combo = blockIdx.x;                 // 0..19
   const int BK = kBK[dt][combo / 10];
   const int s = 2 + (combo / 2) % 5;
   const int g = 1 + combo % 2;
-  const float W = grouped_working_set<float>(Mg, G, N, K, dt);
+  for (int q = threadIdx.x; q < G; q += blockDim.x) Ms[q] = Mg[q];
+  __syncthreads();
+  const float W = grouped_working_set<float>(Ms, G, N, K, dt);
   bool any_invalid = false;
-  for (int q = threadIdx.x; q < G; q += blockDim.x) {
-    float best = INFINITY;
-    int bm = 0, bn = 0;
-    float btau = 0.f;
-    int64_t btiles = 0;
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b) {
-        const int BM = kBM[a], BN = kBN[b];
-        if (!tile_valid(BM, BN, BK, s, g, dt)) continue;
+  constexpr int kPass = kGroupTuneThreads / 9;  // groups per pass
+  for (int q0 = 0; q0 < G; q0 += kPass) {
+    const int t = (int)threadIdx.x;
+    const int q = q0 + t / 9, a = (t % 9) / 3, b = t % 3;
+    if (t < 9 * kPass && q < G) {
+      float cost = INFINITY, tq = 0.f;
+      const int BM = kBM[a], BN = kBN[b];
+      if (tile_valid(BM, BN, BK, s, g, dt)) {
         pm_cfg c;
-        c.M = Mg[q]; c.N = N; c.K = K; c.BM = (int16_t)BM; c.BN = (int16_t)BN; c.BK = (int16_t)BK;
+        c.M = Ms[q]; c.N = N; c.K = K; c.BM = (int16_t)BM; c.BN = (int16_t)BN; c.BK = (int16_t)BK;
         c.stages = (int8_t)s; c.cta_group = (int8_t)g; c.dtype = (int8_t)dt; c.kind = 0; c.tmem_a = 0;
         GemmFwd f;
         gemm_forward(c, th, n_sm, f, W);
-        const float tq = f.Kt * f.T_step + f.T_store;   // one tile of this group
-        const int64_t nt = launch_tiles(th, c.M, N, BM, BN, g);
-        const float cost = (float)nt * tq;
-        if (cost < best) { best = cost; bm = BM; bn = BN; btau = tq; btiles = nt; }
+        tq = f.Kt * f.T_step + f.T_store;                // one tile of this group
+        cost = (float)launch_tiles(th, c.M, N, BM, BN, g) * tq;
       }
-    if (best == INFINITY) any_invalid = true;
-    // each group's own tile decides its buffering here; the launch's rule is
-    // applied below
-    tau[q] = btau;
-    tiles[q] = btiles;
-    bm_s[q] = (int16_t)bm;
-    bn_s[q] = (int16_t)bn;
-    out_bm[combo * G + q] = (int16_t)bm;
-    out_bn[combo * G + q] = (int16_t)bn;
+      cand_cost[t] = cost;
+      cand_tau[t] = tq;
+    }
+    __syncthreads();
+    const int p = q0 + t;
+    if (t < kPass && p < G) {
+      float best = INFINITY;
+      int pick = -1;
+#pragma unroll
+      for (int k = 0; k < 9; ++k)
+        if (cand_cost[9 * t + k] < best) { best = cand_cost[9 * t + k]; pick = k; }
+      if (pick < 0) any_invalid = true;
+      // each group's own tile decides its buffering here; the launch's rule is
+      // applied below
+      const int bm = pick < 0 ? 0 : kBM[pick / 3], bn = pick < 0 ? 0 : kBN[pick % 3];
+      tau[p] = pick < 0 ? 0.f : cand_tau[9 * t + pick];
+      tiles[p] = pick < 0 ? 0 : launch_tiles(th, Ms[p], N, bm, bn, g);
+      bm_s[p] = (int16_t)bm;
+      bn_s[p] = (int16_t)bn;
+      out_bm[combo * G + p] = (int16_t)bm;
+      out_bn[combo * G + p] = (int16_t)bn;
+    }
+    __syncthreads();
   }
   any_invalid = __syncthreads_or(any_invalid);
   // the launch keeps one accumulator buffer if any group's tile needs it
@@ -891,8 +986,11 @@ __global__ void __launch_bounds__(kGroupThreads) grouped_tune_kernel(const int32
       if (bm_s[q] > 0 && !single_buffer(bm_s[q], bn_s[q], BK, s, g, dt, 0))
         tau[q] += 4.0f * (float)bm_s[q] * (float)bn_s[q] * th.inv[17];
   __syncthreads();
-  grouped_list(bm_s, bn_s, tiles, G, list, off);
-  const float t = grouped_makespan<float>(tau, list, off, G, g == 1 ? n_sm : 2 * (n_sm / 2), nullptr);
+  const int64_t n_conc = g == 1 ? n_sm : 2 * (n_sm / 2);
+  grouped_list(bm_s, bn_s, tiles, G, n_conc, sc);
+  for (int q = threadIdx.x; q < G; q += blockDim.x) sc.tau[sc.pos[q]] = tau[q];
+  __syncthreads();
+  const float t = grouped_makespan(sc, G, n_conc, nullptr);
   if (threadIdx.x == 0)
     out_t[combo] = (any_invalid || (g != 1 && n_sm < 2)) ? INFINITY : launch_time(th) + t;
 }
@@ -908,45 +1006,53 @@ __global__ void __launch_bounds__(kGroupThreads) grouped_predict_kernel(const in
                                                                         int K, int BK, int s, int g, int dt,
                                                                         ThetaT<F> th, int n_sm, bool grad,
                                                                         F* __restrict__ out) {
-  __shared__ F tau[kMaxGroups];
+  __shared__ Schedule<F> sc;
   __shared__ int64_t tiles[kMaxGroups];
-  __shared__ int64_t off[kMaxGroups + 1];
-  __shared__ int16_t list[kMaxGroups], pos[kMaxGroups];
+  __shared__ int32_t Ms[kMaxGroups];
+  __shared__ int16_t bm_s[kMaxGroups], bn_s[kMaxGroups];
   __shared__ F red_d[kGroupThreads / 32][NP];
-  const F W = grouped_working_set<F>(Mg, G, N, K, dt);
+  for (int q = threadIdx.x; q < G; q += blockDim.x) {
+    Ms[q] = Mg[q];
+    bm_s[q] = BMg[q];
+    bn_s[q] = BNg[q];
+  }
+  __syncthreads();
+  const F W = grouped_working_set<F>(Ms, G, N, K, dt);
   const int64_t n_conc = g == 1 ? n_sm : 2 * (n_sm / 2);
   // one accumulator buffer for the whole launch if any group's tile needs it
   bool single = false;
-  for (int q = threadIdx.x; q < G; q += blockDim.x) single = single || single_buffer(BMg[q], BNg[q], BK, s, g, dt, 0);
-  const int sb = __syncthreads_or(single) ? 1 : 0;
   for (int q = threadIdx.x; q < G; q += blockDim.x) {
+    single = single || single_buffer(bm_s[q], bn_s[q], BK, s, g, dt, 0);
+    tiles[q] = launch_tiles(th, Ms[q], N, bm_s[q], bn_s[q], g);
+  }
+  const int sb = __syncthreads_or(single) ? 1 : 0;
+  grouped_list(bm_s, bn_s, tiles, G, n_conc, sc);
+  auto group_cfg = [&](int q) {
     pm_cfg c;
-    c.M = Mg[q]; c.N = N; c.K = K; c.BM = BMg[q]; c.BN = BNg[q]; c.BK = (int16_t)BK;
+    c.M = Ms[q]; c.N = N; c.K = K; c.BM = bm_s[q]; c.BN = bn_s[q]; c.BK = (int16_t)BK;
     c.stages = (int8_t)s; c.cta_group = (int8_t)g; c.dtype = (int8_t)dt; c.kind = 0; c.tmem_a = 0;
+    return c;
+  };
+  for (int q = threadIdx.x; q < G; q += blockDim.x) {
     GemmFwdT<F> f;
-    gemm_forward(c, th, n_sm, f, W, sb);
-    tau[q] = f.Kt * f.T_step + f.T_store;
-    tiles[q] = launch_tiles(th, c.M, N, c.BM, c.BN, g);
+    gemm_forward(group_cfg(q), th, n_sm, f, W, sb);
+    sc.tau[sc.pos[q]] = f.Kt * f.T_step + f.T_store;
   }
   __syncthreads();
-  grouped_list(BMg, BNg, tiles, G, list, off);
   int w_star = 0;
-  const F t = grouped_makespan<F>(tau, list, off, G, n_conc, &w_star);
+  const F t = grouped_makespan(sc, G, n_conc, &w_star);
   const bool none = g != 1 && n_sm < 2;
   if (threadIdx.x == 0) out[0] = none ? (F)__int_as_float(0x7fc00000) : launch_time(th) + t;
   if (!grad) return;
-  for (int i = threadIdx.x; i < G; i += blockDim.x) pos[list[i]] = (int16_t)i;
-  __syncthreads();
   // d T_hat = d launch + sum_q n_{w*,q} d tau_q
   F d[NP];
 #pragma unroll
   for (int j = 0; j < NP; ++j) d[j] = F(0);
   for (int q = threadIdx.x; q < G; q += blockDim.x) {
-    const int64_t cnt = dealt(off[pos[q]], off[pos[q] + 1], w_star, n_conc, G > 1);
+    const int i = sc.pos[q];
+    const int64_t cnt = dealt_before(sc, i + 1, w_star, n_conc, G > 1) - dealt_before(sc, i, w_star, n_conc, G > 1);
     if (!cnt) continue;
-    pm_cfg c;
-    c.M = Mg[q]; c.N = N; c.K = K; c.BM = BMg[q]; c.BN = BNg[q]; c.BK = (int16_t)BK;
-    c.stages = (int8_t)s; c.cta_group = (int8_t)g; c.dtype = (int8_t)dt; c.kind = 0; c.tmem_a = 0;
+    const pm_cfg c = group_cfg(q);
     GemmFwdT<F> f;
     gemm_forward(c, th, n_sm, f, W, sb);
     F gR = F(0), gS = F(0);
@@ -1090,6 +1196,38 @@ extern "C" pm_status pm_autotune_topk(const int32_t* MNK_dev, int64_t n, int32_t
 
 namespace pm {
 
+// Page-locked host memory of the grouped model calls, one block per calling
+// thread: the kernels read the row counts and tiles from it and write their
+// results to it, so a call is one launch and one wait.  Device scratch from the
+// stream's pool and four copies cost about 270 us a call (the pool gives its
+// memory back at every wait and maps it again).  A call waits for its kernel
+// before it returns, so the block is never in use by two calls; it is given
+// back when the thread ends and by pm_shutdown.
+constexpr size_t kGroupScratch = 4 * kMaxGroups + 2 * 2 * 20 * kMaxGroups + 512;
+
+struct GroupScratch {
+  char* p = nullptr;
+  void release() {
+    if (p) cudaFreeHost(p);
+    p = nullptr;
+  }
+  ~GroupScratch() { release(); }
+};
+static thread_local GroupScratch g_group_scratch;
+
+void release_group_scratch_this_thread() { g_group_scratch.release(); }
+
+static pm_status group_scratch(char** out) {
+  GroupScratch& g = g_group_scratch;
+  if (!g.p) {
+    void* p = nullptr;
+    PM_CUDA(cudaHostAlloc(&p, kGroupScratch, cudaHostAllocPortable | cudaHostAllocMapped));
+    g.p = static_cast<char*>(p);
+  }
+  *out = g.p;
+  return PM_OK;
+}
+
 // All 20 launch-level candidates (BK, stages, cta_group) of the grouped
 // autotuner: predicted makespan ht[i] and per-group tiles hbm/hbn[i * G + q].
 static pm_status grouped_candidates(int32_t G, const int32_t* M_host, int32_t N, int32_t K, int32_t dtype,
@@ -1099,31 +1237,22 @@ static pm_status grouped_candidates(int32_t G, const int32_t* M_host, int32_t N,
   PM_REQUIRE(M_host && theta_host && n_sm > 0, PM_EINVAL, "null pointer or n_sm <= 0");
   PM_REQUIRE(N > 0 && K > 0 && dtype >= 0 && dtype <= 2, PM_EINVAL, "bad N, K or dtype");
   for (int q = 0; q < G; ++q) PM_REQUIRE(M_host[q] > 0, PM_EINVAL, "M[%d] <= 0", q);
-  // device scratch: M (G int32), t (20 floats), bm/bn (20 x G int16 each)
-  const size_t bytes = 256 + G * 4 + 20 * 4 + 2 * 20 * (size_t)G * 2 + 16;
   char* buf = nullptr;
-  PM_CUDA(cudaMallocAsync((void**)&buf, bytes, s));
-  int32_t* dM = (int32_t*)buf;
-  float* dt = (float*)(buf + ((G * 4 + 15) & ~15));
-  int16_t* dbm = (int16_t*)((char*)dt + 96);
-  int16_t* dbn = dbm + 20 * G;
-  hbm.assign(20 * (size_t)G, 0);
-  hbn.assign(20 * (size_t)G, 0);
-  pm_status st = PM_OK;
-  cudaError_t e = cudaMemcpyAsync(dM, M_host, G * 4, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) {
-    grouped_tune_kernel<<<20, kGroupThreads, 0, s>>>(dM, G, N, K, dtype, to_theta(theta_host, n_sm), n_sm, dt, dbm, dbn);
-    st = launch_status("grouped_tune_kernel");
-    if (st == PM_OK) e = cudaMemcpyAsync(ht, dt, 20 * sizeof(float), cudaMemcpyDeviceToHost, s);
-    if (st == PM_OK && e == cudaSuccess)
-      e = cudaMemcpyAsync(hbm.data(), dbm, hbm.size() * 2, cudaMemcpyDeviceToHost, s);
-    if (st == PM_OK && e == cudaSuccess)
-      e = cudaMemcpyAsync(hbn.data(), dbn, hbn.size() * 2, cudaMemcpyDeviceToHost, s);
-  }
-  cudaFreeAsync(buf, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  pm_status st = group_scratch(&buf);
   if (st != PM_OK) return st;
-  if (e != cudaSuccess) return cuda_fail(e, "grouped autotune copies");
+  float* pt = reinterpret_cast<float*>(buf);                    // 20 floats
+  int32_t* pM = reinterpret_cast<int32_t*>(buf + 128);          // G
+  int16_t* pbm = reinterpret_cast<int16_t*>(pM + G);            // 20 x G each
+  int16_t* pbn = pbm + 20 * (size_t)G;
+  std::copy(M_host, M_host + G, pM);
+  grouped_tune_kernel<<<20, kGroupTuneThreads, 0, s>>>(pM, G, N, K, dtype, to_theta(theta_host, n_sm), n_sm, pt, pbm,
+                                                       pbn);
+  st = launch_status("grouped_tune_kernel");
+  if (st != PM_OK) return st;
+  PM_CUDA(cudaStreamSynchronize(s));
+  std::copy(pt, pt + 20, ht);
+  hbm.assign(pbm, pbm + 20 * (size_t)G);
+  hbn.assign(pbn, pbn + 20 * (size_t)G);
   return PM_OK;
 }
 
@@ -1155,26 +1284,21 @@ static pm_status grouped_eval(int32_t G, const int32_t* M_host, int32_t N, int32
   }
   const int n_out = grad ? 1 + NP : 1;
   char* buf = nullptr;
-  const size_t bytes = 256 + (size_t)G * 8 + 16 + (size_t)n_out * sizeof(F);
-  PM_CUDA(cudaMallocAsync((void**)&buf, bytes, s));
-  int32_t* dM = (int32_t*)buf;
-  int16_t* dbm = (int16_t*)(buf + ((G * 4 + 15) & ~15));
-  int16_t* dbn = dbm + ((G + 7) & ~7);
-  F* dt = (F*)(dbn + ((G + 7) & ~7));
-  pm_status st = PM_OK;
-  cudaError_t e = cudaMemcpyAsync(dM, M_host, G * 4, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dbm, BM_host, G * 2, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dbn, BN_host, G * 2, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) {
-    grouped_predict_kernel<F><<<1, kGroupThreads, 0, s>>>(dM, dbm, dbn, G, N, K, BK, stages, cta_group, dtype, th,
-                                                           n_sm, grad, dt);
-    st = launch_status("grouped_predict_kernel");
-    if (st == PM_OK) e = cudaMemcpyAsync(out_host, dt, n_out * sizeof(F), cudaMemcpyDeviceToHost, s);
-  }
-  cudaFreeAsync(buf, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  pm_status st = group_scratch(&buf);
   if (st != PM_OK) return st;
-  if (e != cudaSuccess) return cuda_fail(e, "grouped predict copies");
+  F* pt = reinterpret_cast<F*>(buf);                            // 1 + NP values
+  int32_t* pM = reinterpret_cast<int32_t*>(buf + 256);          // G each
+  int16_t* pbm = reinterpret_cast<int16_t*>(pM + G);
+  int16_t* pbn = pbm + G;
+  std::copy(M_host, M_host + G, pM);
+  std::copy(BM_host, BM_host + G, pbm);
+  std::copy(BN_host, BN_host + G, pbn);
+  grouped_predict_kernel<F><<<1, kGroupThreads, 0, s>>>(pM, pbm, pbn, G, N, K, BK, stages, cta_group, dtype, th, n_sm,
+                                                         grad, pt);
+  st = launch_status("grouped_predict_kernel");
+  if (st != PM_OK) return st;
+  PM_CUDA(cudaStreamSynchronize(s));
+  std::copy(pt, pt + n_out, out_host);
   return PM_OK;
 }
 
