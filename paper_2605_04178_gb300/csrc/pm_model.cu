@@ -172,7 +172,7 @@ __host__ __device__ inline bool single_buffer(int BM, int BN, int BK, int s, int
 template <class F>
 struct GemmFwdT {
   F T, T_stage, T_rl, A_rl, B_rl;
-  F T_c, T_io, T_tma, oma, X, R, S, invR, invS, T_step, T_store;
+  F T_c, T_io, T_tma, oma, X, XT, R, S, invR, invS, T_step, T_store;   // XT: T_c without T_mgmt/K_tiles
   F D, DA_r, DA_w, bstep, store_bytes, n_instr;
   F waves, Kt;
   F W, E, rho;          // L2 residency of the TMA loads (measured reading)
@@ -183,6 +183,18 @@ struct GemmFwdT {
   bool drain;           // measured reading, one accumulator buffer: each tile's drain is paid
 };
 using GemmFwd = GemmFwdT<float>;
+
+// Waves of `tiles` CTA tiles over the concurrent CTAs of cta_group g (pairs on
+// fewer than two SMs are rejected by the callers; the guard keeps the division
+// defined).
+template <class F>
+__device__ __forceinline__ int64_t wave_count(int64_t tiles, int g, const ThetaT<F>& th, int n_sm) {
+  if (th.nc_nsm == n_sm && (uint64_t)tiles < 0x80000000ull) {
+    const UDiv u = g == 1 ? th.nc[0] : th.nc[1];
+    return (int64_t)udiv((uint32_t)tiles + (u.d - 1u), u);
+  }
+  return cdiv(tiles, g == 1 ? n_sm : (n_sm >= 2 ? 2 * (n_sm / 2) : 1));
+}
 
 // Stage-centric GEMM time:
 //   T_TMEM = (D + D_A,r)/BW_rd + n_instr L_mma + (D + D_A,w)/BW_wr   (Eq. 2)
@@ -229,16 +241,7 @@ __device__ __forceinline__ void gemm_forward(const pm_cfg& c, const ThetaT<F>& t
   // CTA tiles: ceil(M/BM) ceil(N/BN) (literal); a pair covers 2 BM x BN (measured)
   const int64_t tiles = measured ? (int64_t)g * cdiv(c.M, (int64_t)g * c.BM) * cdiv(c.N, c.BN)
                                  : cdiv(c.M, c.BM) * cdiv(c.N, c.BN);
-  // (pairs on fewer than two SMs are rejected by the callers; the guard keeps
-  // the division defined)
-  const int64_t n_conc = g == 1 ? n_sm : (n_sm >= 2 ? 2 * (n_sm / 2) : 1);
-  int64_t waves;
-  if (th.nc_nsm == n_sm && (uint64_t)tiles < 0x80000000ull) {
-    const UDiv u = g == 1 ? th.nc[0] : th.nc[1];
-    waves = (int64_t)udiv((uint32_t)tiles + (u.d - 1u), u);
-  } else {
-    waves = cdiv(tiles, n_conc);
-  }
+  const int64_t waves = wave_count(tiles, g, th, n_sm);
   f.Kt = count_to<F>(Kt);
   f.waves = count_to<F>(waves);
   // tile products in integers (exact: at most 2^25), one conversion each
@@ -257,7 +260,8 @@ __device__ __forceinline__ void gemm_forward(const pm_cfg& c, const ThetaT<F>& t
   f.invS = g == 1 ? F(1) : th.inv[14];
   const int rows = (measured && g == 1 && c.BM < 128) ? 128 : (int)c.BM;
   f.X = (np * (F)(2 * rows * (int)c.BN * (int)c.BK)) * (f.invR * f.invS);
-  f.T_c = f.X + T_tmem + T_mgmt;
+  f.XT = f.X + T_tmem;
+  f.T_c = f.XT + T_mgmt;
   // BN / g: exact for the one- and two-SM tiles (power-of-two BN)
   const F bn_g = g == 1 ? (F)c.BN : (g == 2 ? F(0.5) * (F)c.BN : (F)c.BN / (F)g);
   f.bstep = g <= 2 ? l * e * (F)((int)c.BK * ((int)c.BM + ((int)c.BN >> (g - 1))))
@@ -584,9 +588,27 @@ static int grad_blocks(int64_t n) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(want, cap));
 }
 
-// Autotuner: one block per shape, thread t evaluates tile configuration t of
-// the 180-point space in lexicographic (BM, BN, BK, stages, cta_group) order.
-constexpr int kTuneThreads = 192;
+// Autotuner: the k predicted-fastest valid configurations of each shape over
+// the 180-point space in lexicographic (BM, BN, BK, stages, cta_group) order,
+// in increasing predicted time, ties to the first.  Two splits of the work with
+// the same results, bit for bit:
+//
+// autotune_table_kernel (many shapes): a block tabulates the terms of Eqs. 2-8
+// that depend on the tile only, for the valid tiles of the type, once; then a
+// warp takes a shape: its lanes work out the shape's terms (bytes, rho, the
+// roofline bounds, one wave count per cta_group, BM and BN) and evaluate up to
+// six tiles each from the table with the arithmetic of gemm_forward.  Bound:
+// ALU issue; BF16 (121 valid tiles), best tile of 5,556 shapes 17.1 -> 7.0 us and
+// of 555,555 shapes 1385 -> 352 us against a whole model evaluation per
+// (shape, tile); best eight of 5,556 shapes 47.1 -> 14.0 us.
+//
+// autotune_shape_kernel (few shapes): a block per shape, thread t evaluates
+// tile t.  Bound: latency; it has no table to build before the first shape, so
+// it is the faster one while every block is resident at once (launch_autotune).
+constexpr int kTuneThreads = 512;
+constexpr int kTuneTiles = 180;
+constexpr int kTunePerLane = (kTuneTiles + 31) / 32;
+constexpr int kMaxTopK = 16;
 
 __device__ __forceinline__ void decode_tile(int t, int dt, int& BM, int& BN, int& BK, int& s, int& g) {
   BM = kBM[t / 60];
@@ -596,126 +618,183 @@ __device__ __forceinline__ void decode_tile(int t, int dt, int& BM, int& BN, int
   g = 1 + t % 2;
 }
 
-__global__ void __launch_bounds__(kTuneThreads) autotune_kernel(const int32_t* __restrict__ MNK, int64_t n, int dt,
-                                                                Theta th, int n_sm, pm_cfg* __restrict__ picks,
-                                                                float* __restrict__ t_pred) {
-  __shared__ float sv[kTuneThreads / 32];
-  __shared__ int si[kTuneThreads / 32];
-  const int t = threadIdx.x;
-  for (int64_t shape = blockIdx.x; shape < n; shape += gridDim.x) {
-    pm_cfg c;
-    c.M = __ldg(MNK + 3 * shape);
-    c.N = __ldg(MNK + 3 * shape + 1);
-    c.K = __ldg(MNK + 3 * shape + 2);
-    c.dtype = (int8_t)dt;
-    c.kind = PM_KIND_GEMM;
-    c.tmem_a = 0;
-    float v = INFINITY;
-    int BM = 0, BN = 0, BK = 0, s = 0, g = 0;
-    if (t < 180) {
-      decode_tile(t, dt, BM, BN, BK, s, g);
-      if (tile_valid(BM, BN, BK, s, g, dt) && (g == 1 || n_sm >= 2) && c.M > 0 && c.N > 0 && c.K > 0) {
-        c.BM = (int16_t)BM; c.BN = (int16_t)BN; c.BK = (int16_t)BK;
-        c.stages = (int8_t)s; c.cta_group = (int8_t)g;
-        GemmFwd f;
-        gemm_forward(c, th, n_sm, f);
-        v = f.T;
-      }
-    }
-    // argmin, ties to the lower index
-    int idx = t;
+// The tile's wave-count slot (cta_group, BM, BN) and BK index.
+__device__ __forceinline__ int tile_slot(int t) { return (t % 2) * 9 + (t / 60) * 3 + (t / 20) % 3; }
+__device__ __forceinline__ int tile_bk(int t) { return (t / 10) % 2; }
+
+// k rounds of warp argmin over (time, index): lane l holds the times of the
+// candidates l, l + 32, ... in v (INFINITY where there is none).  Lane r < k gets
+// round r's time and index (-1: no candidate left).  A NaN time loses to any
+// finite one.
+__device__ __forceinline__ void warp_topk(float (&v)[kTunePerLane], int k, float& my_t, int& my_i) {
+  const int lane = threadIdx.x & 31;
+  my_t = INFINITY;
+  my_i = -1;
+  for (int r = 0; r < k; ++r) {
+    float bv = v[0];
+    int bi = lane;
+#pragma unroll
+    for (int j = 1; j < kTunePerLane; ++j)
+      if (v[j] < bv || (bv != bv && v[j] < INFINITY)) { bv = v[j]; bi = lane + 32 * j; }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      const float ov = __shfl_xor_sync(0xffffffffu, v, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-      if (ov < v || (ov == v && oi < idx)) { v = ov; idx = oi; }
+      const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ov < bv || (ov == bv && oi < bi) || (bv != bv && ov < INFINITY)) { bv = ov; bi = oi; }
     }
-    if ((t & 31) == 0) { sv[t >> 5] = v; si[t >> 5] = idx; }
-    __syncthreads();
-    if (t == 0) {
-      float bv = sv[0];
-      int bi = si[0];
-      for (int w = 1; w < kTuneThreads / 32; ++w)
-        if (sv[w] < bv || (sv[w] == bv && si[w] < bi)) { bv = sv[w]; bi = si[w]; }
-      pm_cfg p = c;
-      if (bv < INFINITY) {
-        decode_tile(bi, dt, BM, BN, BK, s, g);
-        p.BM = (int16_t)BM; p.BN = (int16_t)BN; p.BK = (int16_t)BK;
-        p.stages = (int8_t)s; p.cta_group = (int8_t)g;
-      } else {
-        p.BM = p.BN = p.BK = 0; p.stages = p.cta_group = 0;
-      }
-      picks[shape] = p;
-      t_pred[shape] = bv;
-    }
-    __syncthreads();
+    bv = __shfl_sync(0xffffffffu, bv, 0);
+    bi = __shfl_sync(0xffffffffu, bi, 0);
+    if (!(bv < INFINITY)) bi = -1;
+    if (lane == r) { my_t = bv; my_i = bi; }
+#pragma unroll
+    for (int j = 0; j < kTunePerLane; ++j)
+      if (bi == lane + 32 * j) v[j] = INFINITY;
   }
 }
 
-// Top-k variant: the k predicted-fastest valid configurations per shape, in
-// increasing predicted time (ties to the lower index), by k rounds of block
-// argmin over the 180 candidates.
-constexpr int kMaxTopK = 16;
+// The record of tile t (t < 0: none, BM = 0) for a shape.
+__device__ __forceinline__ pm_cfg tune_pick(int M, int N, int K, int dt, int t) {
+  pm_cfg p;
+  p.M = M; p.N = N; p.K = K;
+  p.dtype = (int8_t)dt; p.kind = PM_KIND_GEMM; p.tmem_a = 0;
+  p.BM = p.BN = p.BK = 0; p.stages = p.cta_group = 0;
+  if (t >= 0) {
+    int BM, BN, BK, s, g;
+    decode_tile(t, dt, BM, BN, BK, s, g);
+    p.BM = (int16_t)BM; p.BN = (int16_t)BN; p.BK = (int16_t)BK;
+    p.stages = (int8_t)s; p.cta_group = (int8_t)g;
+  }
+  return p;
+}
 
-__global__ void __launch_bounds__(kTuneThreads) autotune_topk_kernel(const int32_t* __restrict__ MNK, int64_t n,
-                                                                     int dt, Theta th, int n_sm, int k,
-                                                                     pm_cfg* __restrict__ picks,
-                                                                     float* __restrict__ t_pred) {
-  __shared__ float sv[kTuneThreads / 32];
-  __shared__ int si[kTuneThreads / 32];
-  __shared__ int chosen;
-  const int t = threadIdx.x;
-  for (int64_t shape = blockIdx.x; shape < n; shape += gridDim.x) {
-    pm_cfg c;
-    c.M = __ldg(MNK + 3 * shape);
-    c.N = __ldg(MNK + 3 * shape + 1);
-    c.K = __ldg(MNK + 3 * shape + 2);
-    c.dtype = (int8_t)dt;
-    c.kind = PM_KIND_GEMM;
-    c.tmem_a = 0;
-    float mine = INFINITY;
-    int BM = 0, BN = 0, BK = 0, s = 0, g = 0;
-    if (t < 180) {
-      decode_tile(t, dt, BM, BN, BK, s, g);
-      if (tile_valid(BM, BN, BK, s, g, dt) && (g == 1 || n_sm >= 2) && c.M > 0 && c.N > 0 && c.K > 0) {
-        c.BM = (int16_t)BM; c.BN = (int16_t)BN; c.BK = (int16_t)BK;
-        c.stages = (int8_t)s; c.cta_group = (int8_t)g;
-        GemmFwd f;
-        gemm_forward(c, th, n_sm, f);
-        mine = f.T;
+__global__ void __launch_bounds__(kTunePerLane * 32) autotune_shape_kernel(const int32_t* __restrict__ MNK, int64_t n,
+                                                                          int dt, Theta th, int n_sm, int k,
+                                                                          pm_cfg* __restrict__ picks,
+                                                                          float* __restrict__ t_pred) {
+  __shared__ float times[kTunePerLane * 32];
+  const int t = threadIdx.x, lane = t & 31;
+  const int64_t shape = blockIdx.x;
+  pm_cfg c;
+  c.M = __ldg(MNK + 3 * shape);
+  c.N = __ldg(MNK + 3 * shape + 1);
+  c.K = __ldg(MNK + 3 * shape + 2);
+  int BM, BN, BK, s, g;
+  decode_tile(min(t, kTuneTiles - 1), dt, BM, BN, BK, s, g);
+  float time = INFINITY;
+  if (t < kTuneTiles && tile_valid(BM, BN, BK, s, g, dt) && (g == 1 || n_sm >= 2) && c.M > 0 && c.N > 0 && c.K > 0) {
+    c.BM = (int16_t)BM; c.BN = (int16_t)BN; c.BK = (int16_t)BK;
+    c.stages = (int8_t)s; c.cta_group = (int8_t)g; c.dtype = (int8_t)dt; c.kind = PM_KIND_GEMM; c.tmem_a = 0;
+    GemmFwd f;
+    gemm_forward(c, th, n_sm, f);
+    time = f.T;
+  }
+  times[t] = time;
+  __syncthreads();
+  if (t >= 32) return;
+  float v[kTunePerLane], my_t;
+  int my_i;
+#pragma unroll
+  for (int j = 0; j < kTunePerLane; ++j) v[j] = times[lane + 32 * j];
+  warp_topk(v, k, my_t, my_i);
+  if (lane < k) {
+    picks[shape * k + lane] = tune_pick(c.M, c.N, c.K, dt, my_i);
+    t_pred[shape * k + lane] = my_t;
+  }
+}
+
+__global__ void __launch_bounds__(kTuneThreads, 2) autotune_table_kernel(const int32_t* __restrict__ MNK, int64_t n,
+                                                                         int dt, Theta th, int n_sm, int k,
+                                                                         pm_cfg* __restrict__ picks,
+                                                                         float* __restrict__ t_pred) {
+  __shared__ float4 row_a[kTuneTiles];           // T_c (without T_mgmt), b_step / B_TMA, T_store, 1 - alpha
+  __shared__ float2 row_b[kTuneTiles];           // 1 / stages, code: tile | slot << 8 | BK index << 13
+  __shared__ int warp_valid[kTuneThreads / 32];
+  const bool measured = th.reading == PM_READING_MEASURED;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int n_tiles = 0;
+  {
+    const int t = threadIdx.x;
+    int BM, BN, BK, s, g;
+    decode_tile(min(t, kTuneTiles - 1), dt, BM, BN, BK, s, g);
+    const bool valid = t < kTuneTiles && tile_valid(BM, BN, BK, s, g, dt) && (g == 1 || n_sm >= 2);
+    const unsigned vote = __ballot_sync(0xffffffffu, valid);
+    if (lane == 0) warp_valid[warp] = __popc(vote);
+    __syncthreads();
+    int at = __popc(vote & ((1u << lane) - 1u));
+    for (int w = 0; w < (kTuneTiles + 31) / 32; ++w) {
+      if (w < warp) at += warp_valid[w];
+      n_tiles += warp_valid[w];
+    }
+    if (valid) {
+      pm_cfg c;
+      c.M = c.N = c.K = 64;                      // the tabulated terms do not depend on the shape
+      c.BM = (int16_t)BM; c.BN = (int16_t)BN; c.BK = (int16_t)BK;
+      c.stages = (int8_t)s; c.cta_group = (int8_t)g; c.dtype = (int8_t)dt; c.kind = PM_KIND_GEMM; c.tmem_a = 0;
+      GemmFwd f;
+      gemm_forward(c, th, n_sm, f);
+      row_a[at] = make_float4(f.XT, f.bstep * th.inv[5], f.T_store, f.oma);
+      row_b[at] = make_float2(th.inv_s[s], __int_as_float(t | tile_slot(t) << 8 | tile_bk(t) << 13));
+    }
+    __syncthreads();
+  }
+  const float e = dt_bytes(dt), np = dt_passes(dt), l = dt_loads(dt);
+  const int ri = dt_rate(dt);
+  const float T_sync = 2.f * th.v[12];
+  const float launch = measured ? th.v[0] + th.v[13] : th.v[0];
+  const bool blend = measured && th.v[3] > 0.f;
+  for (int64_t shape = (int64_t)blockIdx.x * (kTuneThreads / 32) + warp; shape < n;
+       shape += (int64_t)gridDim.x * (kTuneThreads / 32)) {
+    const int M = __ldg(MNK + 3 * shape), N = __ldg(MNK + 3 * shape + 1), K = __ldg(MNK + 3 * shape + 2);
+    float v[kTunePerLane];
+#pragma unroll
+    for (int j = 0; j < kTunePerLane; ++j) v[j] = INFINITY;
+    if (M > 0 && N > 0 && K > 0) {
+      const float bytes_min = l * e * ((float)M * K + (float)N * K) + 4.f * (float)M * (float)N;
+      const float E = blend ? pm_exp_fast(-bytes_min * th.inv[3]) : 0.f;
+      const float rho = blend ? 1.f + (th.v[16] - 1.f) * E : 1.f;
+      const float flops = np * 2.f * (float)M * (float)N * (float)K;
+      const float B_rl = bytes_min * th.inv[2];
+      float T_rl[2], Kt[2], mgmt[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const float inv_rs = th.inv[ri] * (i == 0 ? 1.f : th.inv[14]);
+        const float A_rl = th.nc_nsm == n_sm ? flops * inv_rs * th.inv_nsm : flops * inv_rs / (float)n_sm;
+        T_rl[i] = launch + (A_rl >= B_rl ? A_rl : B_rl);
+        Kt[i] = count_to<float>(cdiv(K, kBK[dt][i]));
+        mgmt[i] = measured ? 0.f : th.v[13] / Kt[i];
+      }
+      float waves = 0.f;
+      if (lane < 18) {
+        const int g = 1 + lane / 9, BM = kBM[lane % 9 / 3], BN = kBN[lane % 3];
+        const int64_t tiles = measured ? (int64_t)g * cdiv(M, (int64_t)g * BM) * cdiv(N, BN) : cdiv(M, BM) * cdiv(N, BN);
+        waves = count_to<float>(wave_count(tiles, g, th, n_sm));
+      }
+#pragma unroll
+      for (int j = 0; j < kTunePerLane; ++j) {
+        if (32 * j >= n_tiles) break;
+        const int i = min(lane + 32 * j, n_tiles - 1);
+        const float4 a = row_a[i];
+        const float2 b = row_b[i];
+        const int code = __float_as_int(b.y);
+        const float wv = __shfl_sync(0xffffffffu, waves, (code >> 8) & 31);
+        const bool bk1 = (code >> 13) & 1, pair = code & 1;
+        const float T_c = a.x + (bk1 ? mgmt[1] : mgmt[0]);
+        const float T_tma = th.v[4] + (blend ? pm_div_fast(a.y, rho) : a.y);
+        const float T_io = measured ? a.w * T_tma : a.w * T_tma + T_sync;
+        const float T_eq8 = pm_max(T_c, T_io) + T_sync;
+        const float T_ring = measured ? (T_tma + T_c + T_sync) * b.x : 0.f;
+        const float T_step = measured && T_ring > T_eq8 ? T_ring : T_eq8;
+        const float T_stage = launch + wv * ((bk1 ? Kt[1] : Kt[0]) * T_step + a.z);
+        const float bound = pair ? T_rl[1] : T_rl[0];
+        if (lane + 32 * j < n_tiles) v[j] = T_stage >= bound ? T_stage : bound;
       }
     }
-    for (int r = 0; r < k; ++r) {
-      float v = mine;
-      int idx = t;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, v, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-        if (ov < v || (ov == v && oi < idx)) { v = ov; idx = oi; }
-      }
-      if ((t & 31) == 0) { sv[t >> 5] = v; si[t >> 5] = idx; }
-      __syncthreads();
-      if (t == 0) {
-        float bv = sv[0];
-        int bi = si[0];
-        for (int w = 1; w < kTuneThreads / 32; ++w)
-          if (sv[w] < bv || (sv[w] == bv && si[w] < bi)) { bv = sv[w]; bi = si[w]; }
-        pm_cfg p = c;
-        if (bv < INFINITY) {
-          decode_tile(bi, dt, BM, BN, BK, s, g);
-          p.BM = (int16_t)BM; p.BN = (int16_t)BN; p.BK = (int16_t)BK;
-          p.stages = (int8_t)s; p.cta_group = (int8_t)g;
-        } else {
-          p.BM = p.BN = p.BK = 0; p.stages = p.cta_group = 0;
-        }
-        picks[shape * k + r] = p;
-        t_pred[shape * k + r] = bv;
-        chosen = bv < INFINITY ? bi : -1;
-      }
-      __syncthreads();
-      if (t == chosen) mine = INFINITY;
-      __syncthreads();
+    float my_t;
+    int my_i;
+    warp_topk(v, k, my_t, my_i);
+    if (lane < k) {
+      picks[shape * k + lane] = tune_pick(M, N, K, dt, my_i < 0 ? -1 : __float_as_int(row_b[my_i].y) & 255);
+      t_pred[shape * k + lane] = my_t;
     }
   }
 }
@@ -1169,16 +1248,33 @@ extern "C" pm_status pm_model_set_reading(int32_t reading) {
 
 extern "C" int32_t pm_model_reading(void) { return g_reading.load(); }
 
+namespace pm {
+
+static pm_status launch_autotune(const int32_t* MNK, int64_t n, int32_t dtype, const pm_params* theta_host, int32_t n_sm,
+                                 int k, pm_cfg* picks, float* t_pred, cudaStream_t s) {
+  const Theta th = to_theta(theta_host, n_sm);
+  const int64_t sms = std::max(1, sm_count());
+  // measured on 152 SMs, table against block per shape: 900 shapes 4.4 / 4.1 us
+  // (best eight 7.0 / 6.4), 1,200 shapes 4.5 / 4.9 us (7.0 / 7.6)
+  if (n <= 6 * sms) {
+    autotune_shape_kernel<<<(int)n, kTunePerLane * 32, 0, s>>>(MNK, n, dtype, th, n_sm, k, picks, t_pred);
+  } else {
+    constexpr int64_t kWarps = kTuneThreads / 32;
+    const int grid = (int)std::min<int64_t>((n + kWarps - 1) / kWarps, sms * 2);
+    autotune_table_kernel<<<grid, kTuneThreads, 0, s>>>(MNK, n, dtype, th, n_sm, k, picks, t_pred);
+  }
+  return launch_status("autotune_kernel");
+}
+
+}  // namespace pm
+
 extern "C" pm_status pm_autotune_pick(const int32_t* MNK_dev, int64_t n, int32_t dtype, const pm_params* theta_host,
                                       int32_t n_sm, pm_cfg* picks_dev, float* t_pred_dev, void* stream) {
   PM_REQUIRE(n >= 0, PM_EINVAL, "n < 0");
   if (n == 0) return PM_OK;
   PM_REQUIRE(MNK_dev && theta_host && picks_dev && t_pred_dev && n_sm > 0, PM_EINVAL, "null pointer or n_sm <= 0");
   PM_REQUIRE(dtype >= 0 && dtype <= 2, PM_EINVAL, "dtype %d is not a pm_dtype", dtype);
-  const int grid = (int)std::min<int64_t>(n, (int64_t)std::max(1, sm_count()) * 16);
-  autotune_kernel<<<grid, kTuneThreads, 0, static_cast<cudaStream_t>(stream)>>>(
-      MNK_dev, n, dtype, to_theta(theta_host, n_sm), n_sm, picks_dev, t_pred_dev);
-  return launch_status("autotune_kernel");
+  return launch_autotune(MNK_dev, n, dtype, theta_host, n_sm, 1, picks_dev, t_pred_dev, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" pm_status pm_autotune_topk(const int32_t* MNK_dev, int64_t n, int32_t dtype, const pm_params* theta_host,
@@ -1188,10 +1284,7 @@ extern "C" pm_status pm_autotune_topk(const int32_t* MNK_dev, int64_t n, int32_t
   PM_REQUIRE(MNK_dev && theta_host && picks_dev && t_pred_dev && n_sm > 0, PM_EINVAL, "null pointer or n_sm <= 0");
   PM_REQUIRE(dtype >= 0 && dtype <= 2, PM_EINVAL, "dtype %d is not a pm_dtype", dtype);
   PM_REQUIRE(k >= 1 && k <= kMaxTopK, PM_EINVAL, "k must be in [1, %d]", kMaxTopK);
-  const int grid = (int)std::min<int64_t>(n, (int64_t)std::max(1, sm_count()) * 16);
-  autotune_topk_kernel<<<grid, kTuneThreads, 0, static_cast<cudaStream_t>(stream)>>>(
-      MNK_dev, n, dtype, to_theta(theta_host, n_sm), n_sm, k, picks_dev, t_pred_dev);
-  return launch_status("autotune_topk_kernel");
+  return launch_autotune(MNK_dev, n, dtype, theta_host, n_sm, k, picks_dev, t_pred_dev, static_cast<cudaStream_t>(stream));
 }
 
 namespace pm {

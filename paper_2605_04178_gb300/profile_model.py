@@ -6,7 +6,7 @@ The batch is the model-calibration workload: GEMM configurations with shapes
 log-uniform in [16, 16384] rounded to 16, tiles uniform over the 180-point
 space and dtypes uniform (seed 4).  Each round launches, in this order, the
 forward (`model_predict_kernel`), the adjoint (`model_grad_kernel` and its
-FP64 finish kernel) and the autotuner (`autotune_kernel`, the first
+FP64 finish kernel) and the autotuner (`autotune_table_kernel`, the first
 configs/180 shapes over all 180 tiles); `--warmup` untimed rounds, then
 `--reps` timed ones.  Prints the median time of each and the configurations
 per second (CUDA events on the launching stream).

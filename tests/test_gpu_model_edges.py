@@ -52,3 +52,60 @@ def test_grouped_calls_on_streams_and_threads(lib):
     [t.start() for t in th]
     [t.join() for t in th]
     assert got == want
+
+
+# one shape; the last number of shapes that gets a block each and the first that
+# goes through the table (six per SM); one more than the table's warps
+@pytest.mark.parametrize("dt", [0, 1, 2])
+def test_autotune_splits_agree_with_oracle(lib, reading, dt):
+    sms = lib.sm_count()
+    n_all = 32 * sms + 1
+    r = S.splitmix64(41, 3 * n_all).reshape(n_all, 3)
+    MNK = np.where(r[:, :1] % np.uint64(2) == 0, 1 + (r >> np.uint64(50)), 16 * (1 + (r >> np.uint64(54)))).astype(np.int32)
+    MNK[3] = (0, 64, 64)                            # no time for an empty product
+    dev = torch.from_numpy(MNK.ravel()).cuda()
+    idx = np.r_[0:3, 4:64]
+    _, t_o = O.autotune(MNK[idx], dt, THETA, N_SM)
+    whole = None
+    for n in (n_all, 6 * sms + 1, 6 * sms, 1):
+        for k in (1, 16):
+            picks = torch.empty(n * k * 24, dtype=torch.uint8, device="cuda")
+            t = torch.empty(n * k, dtype=torch.float32, device="cuda")
+            lib.pm_autotune_topk(dev, n, dt, THETA, N_SM, k, picks, t)
+            t, picks = t.cpu().numpy().reshape(n, k), picks.cpu().numpy().view(lib.CFG_DTYPE).reshape(n, k)
+            if n > 1:
+                assert np.all(np.abs(t[idx, 0] - t_o) <= 1e-5 * t_o)
+                assert np.all(np.isinf(t[3])) and np.all(picks[3]["BM"] == 0)
+            assert np.all(t[:, 1:] >= t[:, :-1])
+            if k == 16:
+                if whole is None:
+                    whole = (t, picks)
+                # the same numbers whichever way the work is split
+                assert np.array_equal(t.view(np.uint32), whole[0][:n].view(np.uint32))
+                assert picks.tobytes() == whole[1][:n].tobytes()
+            else:
+                first = (t, picks) if n == n_all else first
+                assert picks.tobytes() == first[1][:n].tobytes()
+        one_t = torch.empty(n, dtype=torch.float32, device="cuda")
+        one_p = torch.empty(n * 24, dtype=torch.uint8, device="cuda")
+        lib.pm_autotune_pick(dev, n, dt, THETA, N_SM, one_p, one_t)
+        assert one_p.cpu().numpy().tobytes() == first[1][:n].tobytes()
+
+
+def test_autotune_nan_parameters(lib):
+    # both splits treat times that are not numbers alike: a NaN launch time
+    # leaves no tile, a NaN drain rate leaves the double-buffered ones
+    MNK = torch.tensor([4096, 4096, 4096] * 1000, dtype=torch.int32, device="cuda")
+    for j in (0, 14, 17):
+        th = THETA.copy()
+        th[j] = np.nan
+        got = []
+        for n in (1, 1000):
+            p = torch.empty(n * 24, dtype=torch.uint8, device="cuda")
+            t = torch.empty(n, dtype=torch.float32, device="cuda")
+            lib.pm_autotune_pick(MNK, n, 1, th, N_SM, p, t)
+            rec = p.cpu().numpy().view(lib.CFG_DTYPE)
+            got.append((rec[-1].tobytes(), float(t[-1])))
+            assert np.all(rec["BM"] == 0) == (j == 0)
+            assert bool(torch.isnan(t).all()) == (j == 0)
+        assert got[0][0] == got[1][0] and (j == 0 or got[0][1] == got[1][1])
