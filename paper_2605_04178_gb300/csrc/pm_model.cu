@@ -507,6 +507,35 @@ __device__ __forceinline__ T warp_sum(T v) {
 }
 __device__ __forceinline__ double warp_sum_d(double v) { return warp_sum<double>(v); }
 
+// Sums of N values over the warp's lanes by recursive halving: at every step a
+// lane hands half of its values to its partner and adds the partner's half to
+// the rest, so N = 19 takes 21 shuffles and additions in place of 95.  The tree
+// of each sum is warp_sum's.  One lane ends with the total of value `index`
+// (index < 0: this lane has none).
+template <int C, int O, class T, int N>
+__device__ __forceinline__ void sum_halving(T (&v)[N], int& first, int& mine) {
+  constexpr int H = (C + 1) / 2;
+  const bool up = (threadIdx.x & O) != 0;
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    const T hi = i + H < C ? v[i + H < N ? i + H : 0] : T(0);
+    const T send = up ? v[i] : hi, keep = up ? hi : v[i];
+    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+  }
+  first += up ? H : 0;
+  mine = up ? mine - H : min(mine, H);
+  if constexpr (O > 1) sum_halving<H, O / 2>(v, first, mine);
+}
+
+template <class T, int N>
+__device__ __forceinline__ T warp_sum_each(T (&v)[N], int& index) {
+  static_assert(N <= 32, "one lane per value");
+  int first = 0, mine = N;
+  sum_halving<N, 16>(v, first, mine);
+  index = mine > 0 ? first : -1;
+  return v[0];
+}
+
 // F = float: per-configuration FP32 terms (throughput path); F = double: the
 // whole evaluation in FP64 so the calibration's line searches see a smooth
 // objective.  The FP32 kernel is held to four blocks per SM (64 registers,
@@ -515,16 +544,27 @@ __device__ __forceinline__ double warp_sum_d(double v) { return warp_sum<double>
 template <class F>
 constexpr int grad_min_blocks() { return sizeof(F) == 4 ? 4 : 2; }
 
-template <class F>
-__global__ void __launch_bounds__(kGradThreads, grad_min_blocks<F>()) model_grad_kernel(const pm_cfg* __restrict__ cfgs, int64_t n,
-                                                                  ThetaT<F> th, int n_sm,
-                                                                  const F* __restrict__ t_meas,
-                                                                  double* __restrict__ partials) {
-  F acc[NP];
+// Bound: FP32 ALU issue (10^6 configurations 25.1 -> 22.2 us with the sums by
+// halving; 211 us at 10^7); FP64 at a calibration table's size the latency of one
+// configuration (1,901: 26.8 -> 12.8 us), at 10^6 the FP64 pipe (463 us).
+//
+// One partial record per kGradThreads threads, the threads of a record spread
+// over a cluster of CL blocks: partials[j * records + r] is component j of
+// record r.  CL > 1 for few records, so that they use CL times as many SMs;
+// the sums are the same, term by term, whatever CL.
+template <class F, int CL>
+__global__ void __launch_bounds__(kGradThreads / CL, CL == 1 ? grad_min_blocks<F>() : 1)
+    model_grad_kernel(const pm_cfg* __restrict__ cfgs, int64_t n, const __grid_constant__ ThetaT<F> th, int n_sm,
+                      const F* __restrict__ t_meas, double* __restrict__ partials) {
+  constexpr int kThreads = kGradThreads / CL;
+  asm volatile("griddepcontrol.launch_dependents;");           // the finish kernel may be set up (it waits for this grid)
+  if constexpr (CL > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  const int records = (int)(gridDim.x / CL), rec = (int)(blockIdx.x / CL), part = (int)(blockIdx.x % CL);
+  F acc[NREC];                                   // loss, then the gradient
 #pragma unroll
-  for (int j = 0; j < NP; ++j) acc[j] = F(0);
-  F loss = F(0);
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+  for (int j = 0; j < NREC; ++j) acc[j] = F(0);
+  for (int64_t i = (int64_t)rec * kGradThreads + part * kThreads + threadIdx.x; i < n;
+       i += (int64_t)records * kGradThreads) {
     const pm_cfg c = load_cfg(cfgs + i);
     F d[NP];
 #pragma unroll
@@ -544,44 +584,64 @@ __global__ void __launch_bounds__(kGradThreads, grad_min_blocks<F>()) model_grad
       probe_adjoint(c, th, f, F(1), d);
     }
     const F r = pm_log(T) - pm_log(__ldg(t_meas + i));
-    loss = fma(r, r, loss);
+    acc[0] = fma(r, r, acc[0]);
     const F w = F(2) * r / T;
 #pragma unroll
-    for (int j = 0; j < NP; ++j) acc[j] = fma(w, d[j], acc[j]);
+    for (int j = 0; j < NP; ++j) acc[j + 1] = fma(w, d[j], acc[j + 1]);
   }
   // warp sums in F (FP64 arithmetic is scarce on this GPU), warp totals
-  // combined in FP64
+  // combined in FP64 by the record's first block
   __shared__ double red[kGradThreads / 32][NREC];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  F v = warp_sum<F>(loss);
-  if (lane == 0) red[warp][0] = (double)v;
-#pragma unroll
-  for (int j = 0; j < NP; ++j) {
-    v = warp_sum<F>(acc[j]);
-    if (lane == 0) red[warp][j + 1] = (double)v;
+  int j;
+  const F v = warp_sum_each<F, NREC>(acc, j);
+  const int warp = part * (kThreads / 32) + (threadIdx.x >> 5);
+  if constexpr (CL == 1) {
+    if (j >= 0) red[warp][j] = (double)v;
+    __syncthreads();
+  } else {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // the first block has started
+    if (j >= 0)
+      asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(mapa_shared(smem_u32(&red[warp][j]), 0)), "d"((double)v)
+                   : "memory");
+    __syncwarp();
+    cluster_sync();
+    if (part != 0) return;
   }
-  __syncthreads();
   if (threadIdx.x < NREC) {
     double s = 0.0;
+#pragma unroll
     for (int w = 0; w < kGradThreads / 32; ++w) s += red[w][threadIdx.x];
-    partials[(int64_t)blockIdx.x * NREC + threadIdx.x] = s;
+    partials[(int64_t)threadIdx.x * records + rec] = s;
   }
 }
 
-// Warp j sums component j of the block records: lane l adds records l,
-// l+32, ... in order, then a fixed butterfly combines the lanes, so the
-// result depends only on the number of records (deterministic).
-__global__ void __launch_bounds__(NREC * 32) model_grad_finish_kernel(const double* __restrict__ partials,
-                                                                    int blocks, int64_t n,
-                                                                    double* __restrict__ out) {
-  const int j = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// Block j sums component j of the records: lane l adds records l, l+32, ... in
+// order, then a fixed butterfly combines the lanes, so the result depends only
+// on the number of records (deterministic).  Bound: latency; a block per
+// component reading consecutive records, twenty loads of a lane in flight (608
+// records on 152 SMs), takes 3.7 us where one block with strided records took
+// 8.5, and it is set up while the partial sums are made (programmatic launch:
+// 1.2 to 2.5 us less from one call to the next).
+__global__ void __launch_bounds__(32) model_grad_finish_kernel(const double* __restrict__ partials, int records,
+                                                               int64_t n, double* __restrict__ out) {
+  constexpr int kBatch = 20;
+  asm volatile("griddepcontrol.wait;" ::: "memory");           // the records are complete and visible
+  const double* p = partials + (int64_t)blockIdx.x * records;
   double s = 0.0;
-#pragma unroll 4
-  for (int b = lane; b < blocks; b += 32) s += partials[(int64_t)b * NREC + j];
+  for (int b = threadIdx.x; b < records; b += 32 * kBatch) {
+    double v[kBatch];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) v[u] = b + 32 * u < records ? p[b + 32 * u] : 0.0;
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u)
+      if (b + 32 * u < records) s += v[u];
+  }
   s = warp_sum_d(s);
-  if (lane == 0) out[j] = s / (double)n;
+  if (threadIdx.x == 0) out[blockIdx.x] = s / (double)n;
 }
 
+// Partial records of a call: one per kGradThreads configurations, one wave at most.
 static int grad_blocks(int64_t n) {
   const int64_t want = (n + kGradThreads - 1) / kGradThreads;
   const int cap = std::max(1, sm_count()) * 4;             // one wave: four blocks per SM (launch bound)
@@ -1190,6 +1250,47 @@ extern "C" pm_status pm_model_grad_workspace(int64_t n, size_t* bytes) {
   return PM_OK;
 }
 
+namespace pm {
+
+template <class F>
+static pm_status launch_grad(const pm_cfg* cfgs, int64_t n, const ThetaT<F>& th, int n_sm, const F* t_meas,
+                             double* partials, int records, double* out, cudaStream_t s) {
+  // FP64, few records: a cluster of eight one-warp blocks per record.  Measured
+  // with / without clusters: 1,901 configurations 12.8 / 21.0 us, 20,000 15.9 / 21.3,
+  // 30,000 19.6 / 21.4, 38,000 33.2 / 21.5 (the clusters no longer fit at once).  The
+  // FP32 kernel is bound by one thread's latency and gains nothing.
+  constexpr int CL = sizeof(F) == 8 ? 8 : 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  cfg.attrs = attr;
+  if (CL > 1 && records <= 2 * sm_count() / 3) {
+    cfg.gridDim = dim3((unsigned)records * CL);
+    cfg.blockDim = dim3(kGradThreads / CL);
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = CL;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, model_grad_kernel<F, CL>, cfgs, n, th, n_sm, t_meas, partials);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchKernelEx(model_grad_kernel)");
+  } else {
+    model_grad_kernel<F, 1><<<records, kGradThreads, 0, s>>>(cfgs, n, th, n_sm, t_meas, partials);
+    pm_status st = launch_status("model_grad_kernel");
+    if (st != PM_OK) return st;
+  }
+  cfg.gridDim = dim3(NREC);
+  cfg.blockDim = dim3(32);
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, model_grad_finish_kernel, (const double*)partials, records, n, out);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchKernelEx(model_grad_finish_kernel)");
+  return PM_OK;
+}
+
+}  // namespace pm
+
 extern "C" pm_status pm_model_grad(const pm_cfg* cfgs_dev, int64_t n, const pm_params* theta_host, int32_t n_sm,
                                    const float* t_meas_dev, void* workspace_dev, size_t workspace_bytes,
                                    double* out_dev, void* stream) {
@@ -1203,12 +1304,8 @@ extern "C" pm_status pm_model_grad(const pm_cfg* cfgs_dev, int64_t n, const pm_p
              "workspace of %zu bytes is smaller than the %zu needed", workspace_bytes,
              (size_t)blocks * NREC * sizeof(double));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  model_grad_kernel<float><<<blocks, kGradThreads, 0, s>>>(cfgs_dev, n, to_theta(theta_host, n_sm), n_sm, t_meas_dev,
-                                                           static_cast<double*>(workspace_dev));
-  pm_status st = launch_status("model_grad_kernel");
-  if (st != PM_OK) return st;
-  model_grad_finish_kernel<<<1, NREC * 32, 0, s>>>(static_cast<const double*>(workspace_dev), blocks, n, out_dev);
-  return launch_status("model_grad_finish_kernel");
+  return launch_grad(cfgs_dev, n, to_theta(theta_host, n_sm), n_sm, t_meas_dev, static_cast<double*>(workspace_dev), blocks,
+                     out_dev, s);
 }
 
 extern "C" pm_status pm_model_grad_f64(const pm_cfg* cfgs_dev, int64_t n, const double* theta_host, int32_t n_sm,
@@ -1231,12 +1328,7 @@ extern "C" pm_status pm_model_grad_f64(const pm_cfg* cfgs_dev, int64_t n, const 
   th.reading = g_reading.load();
   set_concurrency(th, n_sm);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  model_grad_kernel<double><<<blocks, kGradThreads, 0, s>>>(cfgs_dev, n, th, n_sm, t_meas_dev,
-                                                            static_cast<double*>(workspace_dev));
-  pm_status st = launch_status("model_grad_kernel");
-  if (st != PM_OK) return st;
-  model_grad_finish_kernel<<<1, NREC * 32, 0, s>>>(static_cast<const double*>(workspace_dev), blocks, n, out_dev);
-  return launch_status("model_grad_finish_kernel");
+  return launch_grad(cfgs_dev, n, th, n_sm, t_meas_dev, static_cast<double*>(workspace_dev), blocks, out_dev, s);
 }
 
 extern "C" pm_status pm_model_set_reading(int32_t reading) {
@@ -1607,9 +1699,5 @@ extern "C" pm_status pm_model_grad_noalloc(const pm_cfg* cfgs_dev, int64_t n, co
   PM_REQUIRE(blocks <= kGradStaticRecords, PM_ENOMEM, "%d partial records exceed the %d the array holds", blocks,
              kGradStaticRecords);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  model_grad_kernel<float><<<blocks, kGradThreads, 0, s>>>(cfgs_dev, n, to_theta(theta_host, n_sm), n_sm, t_meas_dev, scratch);
-  st = launch_status("model_grad_kernel");
-  if (st != PM_OK) return st;
-  model_grad_finish_kernel<<<1, NREC * 32, 0, s>>>(scratch, blocks, n, out_dev);
-  return launch_status("model_grad_finish_kernel");
+  return launch_grad(cfgs_dev, n, to_theta(theta_host, n_sm), n_sm, t_meas_dev, scratch, blocks, out_dev, s);
 }

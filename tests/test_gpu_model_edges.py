@@ -109,3 +109,53 @@ def test_autotune_nan_parameters(lib):
             assert np.all(rec["BM"] == 0) == (j == 0)
             assert bool(torch.isnan(t).all()) == (j == 0)
         assert got[0][0] == got[1][0] and (j == 0 or got[0][1] == got[1][1])
+
+
+# one warp of a record, a whole record and one row more, the last number of
+# records that FP64 spreads over clusters (two thirds of the SMs) and one more
+@pytest.mark.parametrize("rows", [1, 31, 33, 256, 257, "clusters", "clusters+1"])
+def test_gradient_record_sizes(lib, rows):
+    limit = 256 * (2 * lib.sm_count() // 3)
+    n = {"clusters": limit, "clusters+1": limit + 1}.get(rows, rows)
+    c = S.model_config_batch(n, seed=50)
+    c["kind"] = np.zeros(n, dtype=np.int32)
+    c["tmem_a"] = np.zeros(n, dtype=np.int32)
+    t_true, gi = O.model_batch(c, THETA, N_SM, grad=True)
+    t_meas = (t_true * np.exp(0.3 * (S.uniform01_f64(51, n) - 0.5))).astype(np.float32).astype(np.float64)
+    L_o, g_o = O.model_loss_grad(c, THETA, N_SM, t_meas)
+    r = np.log(t_true) - np.log(t_meas)
+    scale = (2.0 / n) * np.sum(np.abs(r[:, None] * gi / t_true[:, None]), axis=0)
+    dev = lib.cfg_tensor(c)
+    ws = torch.empty(lib.pm_model_grad_workspace(n) // 8, dtype=torch.float64, device="cuda")
+    out = torch.empty(lib.N_GRAD_OUT, dtype=torch.float64, device="cuda")
+    for _ in range(2):                              # the workspace is written before it is read
+        lib.pm_model_grad_f64(dev, n, THETA, N_SM, torch.from_numpy(t_meas).cuda(), ws, out)
+        o = out.cpu().numpy()
+        assert o[0] == pytest.approx(L_o, rel=1e-10)
+        assert np.all(np.abs(o[1:] - g_o) <= 1e-10 * scale + 1e-300)
+        ws.fill_(float("nan"))
+    lib.pm_model_grad(dev, n, THETA, N_SM, torch.from_numpy(t_meas.astype(np.float32)).cuda(), ws, out)
+    o = out.cpu().numpy()
+    assert o[0] == pytest.approx(L_o, rel=1e-4, abs=1e-9)
+    assert np.all(np.abs(o[1:] - g_o) <= 1e-4 * scale + 1e-30)
+
+
+def test_gradient_in_a_captured_graph(lib):
+    # the two launches of a call, the second set up during the first, replayed
+    n = 3000
+    c = S.model_config_batch(n, seed=52)
+    c["kind"] = np.zeros(n, dtype=np.int32)
+    dev = lib.cfg_tensor(c)
+    t = torch.full((n,), 1e-4, dtype=torch.float64, device="cuda")
+    ws = torch.empty(lib.pm_model_grad_workspace(n) // 8, dtype=torch.float64, device="cuda")
+    want = torch.empty(lib.N_GRAD_OUT, dtype=torch.float64, device="cuda")
+    lib.pm_model_grad_f64(dev, n, THETA, N_SM, t, ws, want)
+    got = torch.zeros_like(want)
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=s):
+        lib.pm_model_grad_f64(dev, n, THETA, N_SM, t, ws, got, stream=s)
+    for _ in range(3):
+        g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(got, want)
