@@ -181,6 +181,7 @@ struct GemmFwdT {
   int ri;
   bool oma_free, blend, ring;
   bool drain;           // measured reading, one accumulator buffer: each tile's drain is paid
+  F inv_s, inv_s1;      // 1 / stages and 1 / (stages - 1) (gemm_forward_space only)
 };
 using GemmFwd = GemmFwdT<float>;
 
@@ -307,16 +308,17 @@ __device__ __forceinline__ void gemm_forward(const pm_cfg& c, const ThetaT<F>& t
 // d[j] += dtau/dtheta_j; the tensor-rate and S_2SM slopes go to gR and gS
 // (the caller adds them to the right entries).  max() passes the gradient
 // to its first argument on ties; the clamp stops it outside (0,1).
-template <class F>
+// SPACE: f is gemm_forward_space's (measured reading, L2 blend on, 2..6 stages).
+template <bool SPACE = false, class F>
 __device__ __forceinline__ void step_store_adjoint(const pm_cfg& c, const ThetaT<F>& th, const GemmFwdT<F>& f,
                                                    F g_step, F g_store, F (&d)[NP], F& gR, F& gS) {
-  const bool measured = th.reading == PM_READING_MEASURED;
+  const bool measured = SPACE || th.reading == PM_READING_MEASURED;
   d[4] += g_store;
   d[5] -= g_store * (f.store_bytes * th.inv[5]) * th.inv[5];
   if (f.drain) d[17] -= g_store * (f.store_bytes * th.inv[17]) * th.inv[17];
   // T_step = max(T_eq8, T_ring); ties to Eq. 8
   const F g_eq8 = f.ring ? F(0) : g_step;
-  const F g_ring = f.ring ? div_stages(g_step, c.stages, th) : F(0);   // per term of the ring's cycle
+  const F g_ring = f.ring ? (SPACE ? g_step * f.inv_s : div_stages(g_step, c.stages, th)) : F(0);   // per term of the ring's cycle
   F g_sync = g_eq8 + g_ring;
   F g_c = g_ring, g_io = F(0);
   if (f.T_c >= f.T_io) g_c += g_eq8; else g_io = g_eq8;
@@ -324,7 +326,8 @@ __device__ __forceinline__ void step_store_adjoint(const pm_cfg& c, const ThetaT
   if (!measured) g_sync += g_io;
   const F g_tma = g_io * f.oma + g_ring;
   if (f.oma_free)
-    d[15] += measured ? div_stages_m1(g_io * f.T_tma, c.stages, th) : div_stages(g_io * f.T_tma, c.stages, th);
+    d[15] += SPACE ? g_io * f.T_tma * f.inv_s1
+                   : (measured ? div_stages_m1(g_io * f.T_tma, c.stages, th) : div_stages(g_io * f.T_tma, c.stages, th));
   d[4] += g_tma;
   const F t_bw = f.blend ? pm_div_fast(f.bstep * th.inv[5], f.rho) : f.bstep * th.inv[5];   // b_step / (B_TMA rho)
   d[5] -= g_tma * t_bw * th.inv[5];
@@ -355,10 +358,10 @@ __device__ __forceinline__ void rate_adjoint(const pm_cfg& c, const GemmFwdT<F>&
 }
 
 // Adjoint of gemm_forward: d[j] += w * dT_hat/dtheta_j.
-template <class F>
+template <bool SPACE = false, class F>
 __device__ __forceinline__ void gemm_adjoint(const pm_cfg& c, const ThetaT<F>& th, const GemmFwdT<F>& f, F w,
                                              F (&d)[NP]) {
-  const bool measured = th.reading == PM_READING_MEASURED;
+  const bool measured = SPACE || th.reading == PM_READING_MEASURED;
   F g_stage = F(0), g_rl = F(0);
   if (f.T_stage >= f.T_rl) g_stage = w; else g_rl = w;
   F gR = F(0), gS = F(0);
@@ -376,8 +379,104 @@ __device__ __forceinline__ void gemm_adjoint(const pm_cfg& c, const ThetaT<F>& t
   }
   // stage branch: launch + waves (K_tiles T_step + T_store)
   d[0] += g_stage;
-  step_store_adjoint(c, th, f, g_stage * f.waves * f.Kt, g_stage * f.waves, d, gR, gS);
+  step_store_adjoint<SPACE>(c, th, f, g_stage * f.waves * f.Kt, g_stage * f.waves, d, gR, gS);
   rate_adjoint(c, f, gR, gS, d);
+}
+
+// The records that the search space and the calibration table are made of take
+// a shorter way to the same values: GEMM records of TMEM strategy A under the
+// measured reading with BM, BN in {64, 128, 256}, BK in {32, 64, 128}, 2..6 stages
+// and extents below 2^20, whose counts fit in 32 bits and whose extents are
+// divided by shifts.  What depends on (dtype, cta_group) or on the stages alone
+// is looked up in shared memory: kernel parameters indexed by a lane's own value
+// are read once per distinct value.  The floating-point operations are
+// gemm_forward's, in its order, so the results are the same bits.
+struct SpaceTables {
+  float4 rate[6];       // by 2 dtype + (cta_group - 1): 1 / (R S), l e, n_p, 1 / R
+  uint4 conc[2];        // by cta_group - 1: the wave division d - 1, m, s1, s2
+  float4 depth[8];      // by stages: 1 - alpha, 1 / s, 1 / (s - 1), 0 < c_alpha / (s - 1) < 1
+  float inv_s2sm[2];    // by cta_group - 1: 1 / S
+};
+
+// Whether the launch's parameters allow the short way (uniform over the launch).
+__device__ __forceinline__ bool space_tables(const Theta& th, int n_sm, SpaceTables& t) {
+  if (threadIdx.x < 6) {
+    const int dt = threadIdx.x >> 1, g = 1 + (threadIdx.x & 1);
+    const float invR = th.inv[dt_rate(dt)], invS = g == 1 ? 1.f : th.inv[14];
+    t.rate[threadIdx.x] = make_float4(invR * invS, dt_loads(dt) * dt_bytes(dt), dt_passes(dt), invR);
+  } else if (threadIdx.x < 8) {
+    const int i = threadIdx.x - 6;
+    t.conc[i] = make_uint4(th.nc[i].d - 1u, th.nc[i].m, (unsigned)th.nc[i].s1, (unsigned)th.nc[i].s2);
+    t.inv_s2sm[i] = i == 0 ? 1.f : th.inv[14];
+  } else if (threadIdx.x < 16) {
+    const int s = threadIdx.x - 8;
+    const float r = th.v[15] * th.inv_s1[s];
+    t.depth[s] = make_float4(r <= 0.f ? 0.f : (r >= 1.f ? 1.f : r), th.inv_s[s], th.inv_s1[s],
+                             r > 0.f && r < 1.f ? 1.f : 0.f);
+  }
+  __syncthreads();
+  return th.reading == PM_READING_MEASURED && th.nc_nsm == n_sm && th.v[3] > 0.f;
+}
+
+__device__ __forceinline__ bool in_space(const pm_cfg& c) {
+  const unsigned tile = (unsigned)(uint16_t)c.BM | (unsigned)(uint16_t)c.BN << 16, bk = (unsigned)(uint16_t)c.BK;
+  // one bit of 64..256 in each half of `tile`, one of 32..128 in bk
+  return c.kind == PM_KIND_GEMM && c.tmem_a == 0 && (unsigned)(c.stages - 2) <= 4u &&
+         (unsigned)(c.cta_group - 1) <= 1u && (unsigned)c.dtype <= 2u && (tile & ~0x01C001C0u) == 0u &&
+         (tile & 0xFFFFu) != 0u && (tile >> 16) != 0u && (tile & (tile - 0x00010001u)) == 0u && (bk & ~0xE0u) == 0u &&
+         bk != 0u && (bk & (bk - 1u)) == 0u && ((unsigned)(c.M - 1) | (unsigned)(c.N - 1) | (unsigned)(c.K - 1)) < (1u << 20);
+}
+
+__device__ __forceinline__ void gemm_forward_space(const pm_cfg& c, const Theta& th, const SpaceTables& tab, GemmFwd& f) {
+  const int gi = c.cta_group - 1, BM = c.BM, BN = c.BN, BK = c.BK;
+  const float4 rt = tab.rate[2 * c.dtype + gi], dp = tab.depth[c.stages];
+  const uint4 nc = tab.conc[gi];
+  const float np = rt.z, le = rt.y, inv_rs = rt.x;
+  const float bytes_min = le * ((float)c.M * c.K + (float)c.N * c.K) + 4.f * (float)c.M * (float)c.N;
+  f.ri = 6 + c.dtype;
+  f.invR = rt.w;
+  f.invS = tab.inv_s2sm[gi];
+  const int kb = BK >> 6;                                        // 32, 64, 128 -> 0, 1, 2
+  const unsigned tm = (unsigned)(c.M + (BM << gi) - 1) >> (6 + (BM >> 7) + gi);
+  const unsigned tn = (unsigned)(c.N + BN - 1) >> (6 + (BN >> 7));
+  const unsigned x = ((tm * tn) << gi) + nc.x;
+  const unsigned q = __umulhi(nc.y, x);
+  f.waves = (float)(int)((q + ((x - q) >> nc.z)) >> nc.w);
+  f.Kt = (float)(int)((unsigned)(c.K + BK - 1) >> (5 + kb));
+  f.D = (float)(4 * BM * BN);
+  const int blocks = 1 + (BM >> 8);
+  f.n_instr = np * (float)((BK >> (3 + c.dtype)) * blocks);
+  f.DA_w = f.DA_r = 0.f;
+  const float T_tmem = f.D * th.inv[10] + f.n_instr * th.v[9] + f.D * th.inv[11];
+  const int rows = gi == 0 ? max(BM, 128) : BM;
+  f.X = (np * (float)(2 * rows * BN * BK)) * inv_rs;
+  f.T_c = f.X + T_tmem;
+  f.bstep = le * (float)(BK * (BM + (BN >> gi)));
+  f.W = bytes_min;
+  f.blend = true;
+  f.E = pm_exp_fast(-f.W * th.inv[3]);
+  f.rho = 1.f + (th.v[16] - 1.f) * f.E;
+  f.T_tma = __fadd_rn(th.v[4], pm_div_fast(f.bstep * th.inv[5], f.rho));   // not fused with the quotient
+  const float T_sync = 2.f * th.v[12];
+  f.oma = dp.x;
+  f.inv_s = dp.y;
+  f.inv_s1 = dp.z;
+  f.oma_free = dp.w != 0.f;
+  f.T_io = f.oma * f.T_tma;
+  f.T_eq8 = pm_max(f.T_c, f.T_io) + T_sync;
+  f.T_ring = (f.T_tma + f.T_c + T_sync) * f.inv_s;
+  f.ring = f.T_ring > f.T_eq8;
+  f.T_step = f.ring ? f.T_ring : f.T_eq8;
+  f.store_bytes = f.D;
+  f.drain = BM == 256 && BN == 256;                              // 512 columns: one accumulator buffer
+  f.T_store = th.v[4] + f.store_bytes * th.inv[5] + (f.drain ? f.store_bytes * th.inv[17] : 0.f);
+  f.launch = th.v[0] + th.v[13];
+  f.T_stage = f.launch + f.waves * (f.Kt * f.T_step + f.T_store);
+  const float flops = np * 2.f * (float)c.M * (float)c.N * (float)c.K;
+  f.A_rl = flops * inv_rs * th.inv_nsm;
+  f.B_rl = bytes_min * th.inv[2];
+  f.T_rl = f.launch + (f.A_rl >= f.B_rl ? f.A_rl : f.B_rl);
+  f.T = f.T_stage >= f.T_rl ? f.T_stage : f.T_rl;
 }
 
 // Memory probes.  Copy/triad through Eq. 16 with W = beta bytes moved;
@@ -471,15 +570,23 @@ __device__ __forceinline__ pm_cfg load_cfg(const pm_cfg* p) {
   return c;
 }
 
-// Six blocks per SM (40 registers, no spills): 48 warps hide the latency of
-// the dependent FP32 chain better than the 40 of the unbounded 47-register
-// build (10-20 % more configurations per second).
+// Bound: ALU issue (210 warp-instructions per 32 configurations in the search
+// space, 377 for any others; 28 bytes each).  10^6 configurations 13.2 -> 8.5 us,
+// 10^7 114 -> 66 us with the short way of gemm_forward_space.  Six blocks per SM
+// (40 registers, no spills): 48 warps hide the latency of the dependent FP32
+// chain better than 40 or, at 32 registers, 64 (10^6: 11.0 us).
 __global__ void __launch_bounds__(256, 6) model_predict_kernel(const pm_cfg* __restrict__ cfgs, int64_t n, Theta th,
                                                             int n_sm, float* __restrict__ out) {
+  __shared__ SpaceTables tab;
+  const bool space = space_tables(th, n_sm, tab);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const pm_cfg c = load_cfg(cfgs + i);
     float t;
-    if (!cfg_sane(c, n_sm)) {
+    if (space && in_space(c)) {
+      GemmFwd f;
+      gemm_forward_space(c, th, tab, f);
+      t = f.T;
+    } else if (!cfg_sane(c, n_sm)) {
       t = __int_as_float(0x7fc00000);
     } else if (c.kind == PM_KIND_GEMM) {
       GemmFwd f;
@@ -545,7 +652,8 @@ template <class F>
 constexpr int grad_min_blocks() { return sizeof(F) == 4 ? 4 : 2; }
 
 // Bound: FP32 ALU issue (10^6 configurations 25.1 -> 22.2 us with the sums by
-// halving; 211 us at 10^7); FP64 at a calibration table's size the latency of one
+// halving, 14.8 us with the short way of gemm_forward_space; 10^7 218 -> 130 us);
+// FP64 at a calibration table's size the latency of one
 // configuration (1,901: 26.8 -> 12.8 us), at 10^6 the FP64 pipe (463 us).
 //
 // One partial record per kGradThreads threads, the threads of a record spread
@@ -560,6 +668,9 @@ __global__ void __launch_bounds__(kGradThreads / CL, CL == 1 ? grad_min_blocks<F
   asm volatile("griddepcontrol.launch_dependents;");           // the finish kernel may be set up (it waits for this grid)
   if constexpr (CL > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   const int records = (int)(gridDim.x / CL), rec = (int)(blockIdx.x / CL), part = (int)(blockIdx.x % CL);
+  __shared__ SpaceTables tab;
+  bool space = false;
+  if constexpr (sizeof(F) == 4) space = space_tables(th, n_sm, tab);
   F acc[NREC];                                   // loss, then the gradient
 #pragma unroll
   for (int j = 0; j < NREC; ++j) acc[j] = F(0);
@@ -570,7 +681,14 @@ __global__ void __launch_bounds__(kGradThreads / CL, CL == 1 ? grad_min_blocks<F
 #pragma unroll
     for (int j = 0; j < NP; ++j) d[j] = F(0);
     F T;
-    if (!cfg_sane(c, n_sm)) {
+    if (space && in_space(c)) {
+      if constexpr (sizeof(F) == 4) {
+        GemmFwd f;
+        gemm_forward_space(c, th, tab, f);
+        T = f.T;
+        gemm_adjoint<true>(c, th, f, F(1), d);
+      }
+    } else if (!cfg_sane(c, n_sm)) {
       T = (F)__int_as_float(0x7fc00000);
     } else if (c.kind == PM_KIND_GEMM) {
       GemmFwdT<F> f;
@@ -1238,7 +1356,12 @@ extern "C" pm_status pm_model_predict(const pm_cfg* cfgs_dev, int64_t n, const p
   PM_REQUIRE(cfgs_dev && theta_host && t_out_dev && n_sm > 0, PM_EINVAL, "null pointer or n_sm <= 0");
   PM_REQUIRE(((uintptr_t)cfgs_dev & 7) == 0, PM_EINVAL, "cfgs_dev must be 8-byte aligned");
   const int64_t want = (n + 255) / 256;
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)std::max(1, sm_count()) * 16));
+  // one resident wave that walks the records up to eight rounds (10^6 records 8.5 us,
+  // 9.2 with 16 blocks per SM); past that smaller shares even out the SMs' speeds
+  // (10^7: 72 against 66 us)
+  const int64_t resident = (int64_t)std::max(1, sm_count()) * 6;
+  const int64_t cap = want <= 8 * resident ? resident : (int64_t)std::max(1, sm_count()) * 16;
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, cap));
   model_predict_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(cfgs_dev, n, to_theta(theta_host, n_sm),
                                                                             n_sm, t_out_dev);
   return launch_status("model_predict_kernel");

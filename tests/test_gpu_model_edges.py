@@ -159,3 +159,46 @@ def test_gradient_in_a_captured_graph(lib):
         g.replay()
     torch.cuda.synchronize()
     assert torch.equal(got, want)
+
+
+def edge_cfgs(n, seed):
+    """Records on both sides of every limit of the model's short way: tile extents, stages and extents inside and
+    just outside the search space, probe kinds and TMEM strategy B."""
+    r = np.random.default_rng(seed)
+    pick = lambda v: r.choice(np.array(v), n)
+    ext = (1, 63, 64, 65, 255, 16384, (1 << 20) - 1, 1 << 20, (1 << 20) + 1, 3000017)
+    c = dict(M=pick(ext), N=pick(ext), K=pick(ext), BM=pick((32, 64, 128, 192, 256, 320, 512)),
+             BN=pick((32, 64, 128, 192, 256, 384, 512)), BK=pick((16, 32, 48, 64, 96, 128, 160, 256)),
+             stages=pick((1, 2, 3, 6, 7, 8)), cta_group=pick((1, 2)), dtype=pick((0, 1, 2)),
+             kind=pick((0, 0, 0, 0, 0, 0, 1, 2, 3)), tmem_a=pick((0, 0, 0, 1)))
+    # strategy B copies A in 32-byte slices: a K-step of part of one is no tile
+    c["tmem_a"][c["BK"] % 32 != 0] = 0
+    return {k: v.astype(np.int32) for k, v in c.items()}
+
+
+def test_short_way_agrees_with_the_general_one(lib, reading):
+    n = 60000
+    c = edge_cfgs(n, 60)
+    t_o, gi = O.model_batch(c, THETA, N_SM, grad=True)
+    dev = lib.cfg_tensor(c)
+    t = torch.empty(n, dtype=torch.float32, device="cuda")
+    lib.pm_model_predict(dev, n, THETA, N_SM, t)
+    assert np.all(np.abs(t.cpu().numpy() - t_o) <= 1e-5 * t_o)
+    t_meas = (t_o * np.exp(0.3 * (S.uniform01_f64(61, n) - 0.5))).astype(np.float32).astype(np.float64)
+    L_o, g_o = O.model_loss_grad(c, THETA, N_SM, t_meas)
+    r = np.log(t_o) - np.log(t_meas)
+    scale = (2.0 / n) * np.sum(np.abs(r[:, None] * gi / t_o[:, None]), axis=0)
+    ws = torch.empty(lib.pm_model_grad_workspace(n) // 8, dtype=torch.float64, device="cuda")
+    out = torch.empty(lib.N_GRAD_OUT, dtype=torch.float64, device="cuda")
+    lib.pm_model_grad(dev, n, THETA, N_SM, torch.from_numpy(t_meas.astype(np.float32)).cuda(), ws, out)
+    o = out.cpu().numpy()
+    assert o[0] == pytest.approx(L_o, rel=1e-4, abs=1e-9)
+    assert np.all(np.abs(o[1:] - g_o) <= 1e-4 * scale + 1e-30)
+    # what the model cannot evaluate stays without a time
+    bad = {f: v.copy() for f, v in c.items()}
+    for f, v in (("M", 0), ("BM", -64), ("stages", 0), ("cta_group", 3), ("dtype", 3), ("kind", 7), ("tmem_a", 2)):
+        bad[f][:] = v
+        lib.pm_model_predict(lib.cfg_tensor(bad), n, THETA, N_SM, t)
+        wrong = np.ones(n, bool) if f in ("M", "kind") else c["kind"] == 0
+        assert np.all(np.isnan(t.cpu().numpy()[wrong])), f
+        bad[f][:] = c[f]
