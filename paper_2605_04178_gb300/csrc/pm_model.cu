@@ -665,7 +665,7 @@ __global__ void __launch_bounds__(kGradThreads / CL, CL == 1 ? grad_min_blocks<F
     model_grad_kernel(const pm_cfg* __restrict__ cfgs, int64_t n, const __grid_constant__ ThetaT<F> th, int n_sm,
                       const F* __restrict__ t_meas, double* __restrict__ partials) {
   constexpr int kThreads = kGradThreads / CL;
-  asm volatile("griddepcontrol.launch_dependents;");           // the finish kernel may be set up (it waits for this grid)
+  grid_dependents_launch();                      // the finish kernel may be set up (it waits for this grid)
   if constexpr (CL > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   const int records = (int)(gridDim.x / CL), rec = (int)(blockIdx.x / CL), part = (int)(blockIdx.x % CL);
   __shared__ SpaceTables tab;
@@ -744,7 +744,7 @@ __global__ void __launch_bounds__(kGradThreads / CL, CL == 1 ? grad_min_blocks<F
 __global__ void __launch_bounds__(32) model_grad_finish_kernel(const double* __restrict__ partials, int records,
                                                                int64_t n, double* __restrict__ out) {
   constexpr int kBatch = 20;
-  asm volatile("griddepcontrol.wait;" ::: "memory");           // the records are complete and visible
+  grid_dependency_wait();                        // the records are complete and visible
   const double* p = partials + (int64_t)blockIdx.x * records;
   double s = 0.0;
   for (int b = threadIdx.x; b < records; b += 32 * kBatch) {

@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(kPrepThreads) amax_kernel(const float* __restr
                                                             unsigned int a_blocks, const float* __restrict__ B,
                                                             int64_t nB, int a_vec, int b_vec,
                                                             unsigned int* __restrict__ amax_bits) {
+  grid_dependents_launch();                      // the conversion may be set up (it waits for this grid)
   const bool is_a = blockIdx.x < a_blocks;
   const float* x = is_a ? A : B;
   const int64_t n = is_a ? nA : nB;
@@ -135,6 +136,8 @@ template <int MODE>
 __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const PrepArgs p) {
   __shared__ float tile[kPrepTile * (kPrepTile + 1)];
   const int tid = threadIdx.x;
+  grid_dependents_launch();                      // a GEMM on these operands may be set up
+  grid_dependency_wait();                        // what the previous kernel of the stream wrote or still read is settled
   // FP8: the amax pass read A then B front to back; walking the blocks from
   // the end finds the part of the matrices that is still in L2
   const unsigned int blk = MODE == PM_FP8E4M3 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
@@ -246,13 +249,20 @@ pm_status launch_prepare(int dt, const float* A, int64_t rows, const float* B, i
                                                                  aligned(B, 16), p.amax);
     pm_status st = launch_status("amax_kernel");
     if (st != PM_OK) return st;
-    prep_kernel<PM_FP8E4M3><<<(unsigned int)blocks, kPrepThreads, 0, s>>>(p);
-  } else if (dt == PM_BF16) {
-    prep_kernel<PM_BF16><<<(unsigned int)blocks, kPrepThreads, 0, s>>>(p);
-  } else {
-    prep_kernel<PM_FP32><<<(unsigned int)blocks, kPrepThreads, 0, s>>>(p);
   }
-  return launch_status("prep_kernel");
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned int)blocks);
+  cfg.blockDim = dim3(kPrepThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  auto kern = dt == PM_FP8E4M3 ? prep_kernel<PM_FP8E4M3> : (dt == PM_BF16 ? prep_kernel<PM_BF16> : prep_kernel<PM_FP32>);
+  cudaError_t e2 = cudaLaunchKernelEx(&cfg, kern, (const PrepArgs)p);
+  if (e2 != cudaSuccess) return cuda_fail(e2, "cudaLaunchKernelEx(prep_kernel)");
+  return PM_OK;
 }
 
 }  // namespace pm
