@@ -80,7 +80,10 @@ struct GemmParams {
   int lo_row_a, lo_row_b;          // row offset of the lo half (three-pass TF32)
   float* C;
   const float* scales;             // FP8: {s_A, s_B}
-  int tma_store;                   // epilogue stages 32x32 chunks in shared memory and stores them by TMA
+  int c_rows;                      // rows of C, all problems
+  int vec;                         // C rows allow 16-byte stores
+  int tma_store;                   // staged 32x32 chunks are stored by TMA (two staging buffers)
+  int staged;                      // 4 KB staging buffers per epilogue warp: 2, 1 or 0
   uint32_t staging_off;            // byte offset of the epilogue staging area after the ring
   Watchdog wd;
 };
@@ -434,8 +437,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     const int q = warp & 3;                               // TMEM lane quarter of this warp
     float scale = 1.f;
     if constexpr (KIND == 2) scale = 1.f / (__ldg(p.scales) * __ldg(p.scales + 1));
-    const bool vec = (p.N & 3) == 0;
-    const uint32_t stage_base = base + p.staging_off;     // two 4 KB staging buffers per epilogue warp
+    const bool vec = p.vec != 0;
+    const uint32_t stage_base = base + p.staging_off;     // the epilogue warps' staging buffers
     uint32_t sb = 0;
     int it = 0;
     int qh = 0;
@@ -472,13 +475,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           tmem_ld_wait();
           const int col0 = ccol0 + 32 * j;
           // TMA store of the warp's 32 x 32 chunk when its rows are 32
-          // consecutive rows inside the problem (layouts 0 and 2)
+          // consecutive rows of the problem, or of the last problem in C (the
+          // tensor map clips rows past the end of C); layouts 0 and 2
           const int chunk_row0 = T.crow0 + m * 128 + (lrow - lane);
-          if (col0 >= p.N) {
-            // the chunk lies past the last column: nothing to write
-          } else if (p.tma_store && T.layout != 1 && chunk_row0 + 32 <= T.crow_end) {
-            const uint32_t sbuf = stage_base + (uint32_t)((q * 2 + (sb & 1)) * 4096);
-            if (lane == 0) bulk_wait_read<1>();          // the buffer's previous store has read it
+          if (col0 >= p.N || chunk_row0 >= T.crow_end) {
+            // the chunk lies past the last column or row: nothing to write
+          } else if (p.staged && !(T.layout == 1 && vec)) {
+            const bool by_tma = p.tma_store && T.layout != 1 &&
+                                (chunk_row0 + 32 <= T.crow_end || T.crow_end == p.c_rows);
+            const uint32_t sbuf = stage_base + (uint32_t)((p.staged * q + (sb & 1)) * 4096);
+            if (lane == 0) bulk_wait_read<1>();          // the buffer's previous TMA store has read it
             __syncwarp();
             const uint32_t rowp = sbuf + (uint32_t)lane * 128u;
 #pragma unroll
@@ -489,13 +495,49 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                            "f"(__uint_as_float(r[4 * v + 2]) * scale), "f"(__uint_as_float(r[4 * v + 3]) * scale)
                            : "memory");
             }
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) {
-              tma_store_2d(&maps.c, sbuf, col0, chunk_row0);
-              bulk_commit();
+            if (by_tma) {
+              fence_proxy_async_smem();
+              __syncwarp();
+              if (lane == 0) {
+                tma_store_2d(&maps.c, sbuf, col0, chunk_row0);
+                bulk_commit();
+              }
+              ++sb;
+            } else {
+              // Row lengths that TMA cannot store, partial chunks, 64-row tiles:
+              // the lanes write along the rows of C, one 128-byte row segment
+              // per store (four where rows are 16-byte multiples) instead of one
+              // element of 32 rows, which cost 32 requests a store and bound the
+              // kernel.  BF16 4096 x 4095 x 256 96 -> 26 us, 4096 x 4095 x 4096 183 -> 118,
+              // 1000 x 1003 x 1040 18.2 -> 11.2, FP8 300 x 2941 x 528 14.7 -> 7.7.
+              __syncwarp();
+              const int rows = min(T.layout == 1 ? 16 : 32, T.crow_end - chunk_row0);
+              float* c0 = p.C + (size_t)chunk_row0 * p.N + col0;
+              if (vec && col0 + 32 <= p.N) {
+                const int c4 = lane & 7;
+                for (int i = lane >> 3; i < rows; i += 4) {
+                  float4 o;
+                  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o.x), "=f"(o.y), "=f"(o.z), "=f"(o.w)
+                               : "r"(sbuf + (uint32_t)(i * 128 + ((c4 ^ (i & 7)) * 16))));
+                  *reinterpret_cast<float4*>(c0 + (size_t)i * p.N + 4 * c4) = o;
+                }
+              } else {
+                // eight rows' loads in flight (rows past the last read the buffer's rest)
+                const bool in = col0 + lane < p.N;
+                const float* sp = reinterpret_cast<const float*>(dsmem + (sbuf - smem_u32(dsmem)));
+                float* cp = c0 + lane;
+                for (int i0 = 0; i0 < rows; i0 += 8) {
+                  float o[8];
+#pragma unroll
+                  for (int u = 0; u < 8; ++u) o[u] = sp[(i0 + u) * 32 + (((lane >> 2) ^ u) << 2) + (lane & 3)];
+#pragma unroll
+                  for (int u = 0; u < 8; ++u)
+                    if (in && i0 + u < rows) cp[(size_t)u * p.N] = o[u];
+                  cp += (size_t)8 * p.N;
+                }
+              }
+              __syncwarp();                              // the next chunk may take the buffer
             }
-            ++sb;
           } else if (rvalid) {
             if (vec && col0 + 32 <= p.N) {
 #pragma unroll
@@ -772,15 +814,21 @@ static pm_status plan_launch(int dt, int cg, int BK, int stages, int tmem_a, int
   p.alloc_cols = cols;
   p.stage_bytes = stage;
   P.smem = (size_t)stages * stage + 1024;
-  // TMA-store epilogue: eight 4 KB staging buffers after the ring, when they fit
+  // epilogue staging after the ring: two 4 KB buffers per warp (which TMA stores
+  // need), or one where no more fits (256 x 64 x 64 BF16, 5 stages, 8000 x 8000 x 512:
+  // 152 -> 124 us, with 7999 columns 465 -> 139); without any, lanes store their rows
   p.staging_off = (uint32_t)stages * stage;
   p.tma_store = 0;
+  p.c_rows = (int)sum_m;
   const bool c_ok = (N % 4) == 0 && ((uintptr_t)C & 15) == 0;
-  if (c_ok && P.smem + 32768 <= (size_t)(232448 - 1024)) {
+  p.vec = c_ok ? 1 : 0;
+  const size_t room = (size_t)(232448 - 1024) - P.smem;
+  p.staged = room >= 32768 ? 2 : (room >= 16384 ? 1 : 0);
+  P.smem += (size_t)p.staged * 16384;
+  if (c_ok && p.staged == 2) {
     pm_status st = cached_tmap(&P.maps.c, C, TMAP_F32, (uint64_t)sum_m, (uint64_t)N, 32u, 32u, 128);
     if (st != PM_OK) return st;
     p.tma_store = 1;
-    P.smem += 32768;
   }
   const int dtcode = dt == PM_BF16 ? TMAP_BF16 : (dt == PM_FP32 ? TMAP_F32 : TMAP_U8);
   int first_m = -1, first_n = -1;
