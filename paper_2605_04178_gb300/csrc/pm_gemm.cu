@@ -278,6 +278,20 @@ __device__ __forceinline__ bool mma_tile(MmaRing& r, const GemmParams& p, const 
   return true;
 }
 
+// One 32 x 32 FP32 chunk into a staging buffer, lane = row, in the 128-byte
+// swizzle that the C tensor map expects (16-byte column v of row i at v ^ (i & 7)).
+__device__ __forceinline__ void stage_chunk(uint32_t sbuf, int lane, const uint32_t (&r)[32], float scale) {
+  const uint32_t rowp = sbuf + (uint32_t)lane * 128u;
+#pragma unroll
+  for (int v = 0; v < 8; ++v) {
+    const uint32_t addr = rowp + (uint32_t)((v ^ (lane & 7)) * 16);
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr),
+                 "f"(__uint_as_float(r[4 * v + 0]) * scale), "f"(__uint_as_float(r[4 * v + 1]) * scale),
+                 "f"(__uint_as_float(r[4 * v + 2]) * scale), "f"(__uint_as_float(r[4 * v + 3]) * scale)
+                 : "memory");
+  }
+}
+
 template <int CG, int KIND, int TA, int MAXG>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     gemm_kernel(const __grid_constant__ TensorMaps maps, const __grid_constant__ GroupTableT<MAXG> g,
@@ -480,64 +494,60 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           const int chunk_row0 = T.crow0 + m * 128 + (lrow - lane);
           if (col0 >= p.N || chunk_row0 >= T.crow_end) {
             // the chunk lies past the last column or row: nothing to write
-          } else if (p.staged && !(T.layout == 1 && vec)) {
-            const bool by_tma = p.tma_store && T.layout != 1 &&
-                                (chunk_row0 + 32 <= T.crow_end || T.crow_end == p.c_rows);
+          } else if (p.tma_store && T.layout != 1 && (chunk_row0 + 32 <= T.crow_end || T.crow_end == p.c_rows)) {
+            const uint32_t sbuf = stage_base + (uint32_t)((q * 2 + (sb & 1)) * 4096);
+            if (lane == 0) bulk_wait_read<1>();          // the buffer's previous store has read it
+            __syncwarp();
+            stage_chunk(sbuf, lane, r, scale);
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+              tma_store_2d(&maps.c, sbuf, col0, chunk_row0);
+              bulk_commit();
+            }
+            ++sb;
+          } else if (p.staged && !(vec && (p.tma_store || T.layout == 1))) {
+            // Row lengths that TMA cannot store and rings without room for its
+            // two buffers: through the warp's staging buffer, so that the lanes
+            // write along the rows of C, one 128-byte row segment per store (four
+            // where rows are 16-byte multiples) instead of one element of 32
+            // rows, which cost 32 requests a store and bound the kernel.  BF16
+            // 4096 x 4095 x 256 96 -> 30 us, 4096 x 4095 x 4096 181 -> 117, 1000 x 1003 x
+            // 1040 17.9 -> 11.2, FP8 300 x 2941 x 528 14.5 -> 8.2.  (Chunks whose rows
+            // allow 16-byte stores are left to the lanes beside TMA and in 64-row
+            // tiles: staging them made the single-buffered 256 x 256 tiles of grouped
+            // launches 2-3 % slower.)
             const uint32_t sbuf = stage_base + (uint32_t)((p.staged * q + (sb & 1)) * 4096);
             if (lane == 0) bulk_wait_read<1>();          // the buffer's previous TMA store has read it
             __syncwarp();
-            const uint32_t rowp = sbuf + (uint32_t)lane * 128u;
-#pragma unroll
-            for (int v = 0; v < 8; ++v) {
-              const uint32_t addr = rowp + (uint32_t)((v ^ (lane & 7)) * 16);
-              asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr),
-                           "f"(__uint_as_float(r[4 * v + 0]) * scale), "f"(__uint_as_float(r[4 * v + 1]) * scale),
-                           "f"(__uint_as_float(r[4 * v + 2]) * scale), "f"(__uint_as_float(r[4 * v + 3]) * scale)
-                           : "memory");
-            }
-            if (by_tma) {
-              fence_proxy_async_smem();
-              __syncwarp();
-              if (lane == 0) {
-                tma_store_2d(&maps.c, sbuf, col0, chunk_row0);
-                bulk_commit();
+            stage_chunk(sbuf, lane, r, scale);
+            __syncwarp();
+            const int rows = min(T.layout == 1 ? 16 : 32, T.crow_end - chunk_row0);
+            float* c0 = p.C + (size_t)chunk_row0 * p.N + col0;
+            if (vec && col0 + 32 <= p.N) {
+              const int c4 = lane & 7;
+              for (int i = lane >> 3; i < rows; i += 4) {
+                float4 o;
+                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o.x), "=f"(o.y), "=f"(o.z), "=f"(o.w)
+                             : "r"(sbuf + (uint32_t)(i * 128 + ((c4 ^ (i & 7)) * 16))));
+                *reinterpret_cast<float4*>(c0 + (size_t)i * p.N + 4 * c4) = o;
               }
-              ++sb;
             } else {
-              // Row lengths that TMA cannot store, partial chunks, 64-row tiles:
-              // the lanes write along the rows of C, one 128-byte row segment
-              // per store (four where rows are 16-byte multiples) instead of one
-              // element of 32 rows, which cost 32 requests a store and bound the
-              // kernel.  BF16 4096 x 4095 x 256 96 -> 26 us, 4096 x 4095 x 4096 183 -> 118,
-              // 1000 x 1003 x 1040 18.2 -> 11.2, FP8 300 x 2941 x 528 14.7 -> 7.7.
-              __syncwarp();
-              const int rows = min(T.layout == 1 ? 16 : 32, T.crow_end - chunk_row0);
-              float* c0 = p.C + (size_t)chunk_row0 * p.N + col0;
-              if (vec && col0 + 32 <= p.N) {
-                const int c4 = lane & 7;
-                for (int i = lane >> 3; i < rows; i += 4) {
-                  float4 o;
-                  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o.x), "=f"(o.y), "=f"(o.z), "=f"(o.w)
-                               : "r"(sbuf + (uint32_t)(i * 128 + ((c4 ^ (i & 7)) * 16))));
-                  *reinterpret_cast<float4*>(c0 + (size_t)i * p.N + 4 * c4) = o;
-                }
-              } else {
-                // eight rows' loads in flight (rows past the last read the buffer's rest)
-                const bool in = col0 + lane < p.N;
-                const float* sp = reinterpret_cast<const float*>(dsmem + (sbuf - smem_u32(dsmem)));
-                float* cp = c0 + lane;
-                for (int i0 = 0; i0 < rows; i0 += 8) {
-                  float o[8];
+              // eight rows' loads in flight (rows past the last read the buffer's rest)
+              const bool in = col0 + lane < p.N;
+              const float* sp = reinterpret_cast<const float*>(dsmem + (sbuf - smem_u32(dsmem)));
+              float* cp = c0 + lane;
+              for (int i0 = 0; i0 < rows; i0 += 8) {
+                float o[8];
 #pragma unroll
-                  for (int u = 0; u < 8; ++u) o[u] = sp[(i0 + u) * 32 + (((lane >> 2) ^ u) << 2) + (lane & 3)];
+                for (int u = 0; u < 8; ++u) o[u] = sp[(i0 + u) * 32 + (((lane >> 2) ^ u) << 2) + (lane & 3)];
 #pragma unroll
-                  for (int u = 0; u < 8; ++u)
-                    if (in && i0 + u < rows) cp[(size_t)u * p.N] = o[u];
-                  cp += (size_t)8 * p.N;
-                }
+                for (int u = 0; u < 8; ++u)
+                  if (in && i0 + u < rows) cp[(size_t)u * p.N] = o[u];
+                cp += (size_t)8 * p.N;
               }
-              __syncwarp();                              // the next chunk may take the buffer
             }
+            __syncwarp();                                // the next chunk may take the buffer
           } else if (rvalid) {
             if (vec && col0 + 32 <= p.N) {
 #pragma unroll
