@@ -173,7 +173,7 @@ template <class F>
 struct GemmFwdT {
   F T, T_stage, T_rl, A_rl, B_rl;
   F T_c, T_io, T_tma, oma, X, XT, R, S, invR, invS, T_step, T_store;   // XT: T_c without T_mgmt/K_tiles
-  F D, DA_r, DA_w, bstep, store_bytes, n_instr;
+  F D, D_r, D_w, bstep, store_bytes, n_instr;   // D_r, D_w: D with strategy B's reads and writes of A
   F waves, Kt;
   F W, E, rho;          // L2 residency of the TMA loads (measured reading)
   F launch;             // T_launch (+ L_alloc + L_dealloc once per launch, measured reading)
@@ -251,11 +251,11 @@ __device__ __forceinline__ void gemm_forward(const pm_cfg& c, const ThetaT<F>& t
   // issues, BK/k_instr per 128-row block per pass (measured)
   const int kin = dt == PM_FP32 ? 8 : (dt == PM_BF16 ? 16 : 32);
   f.n_instr = measured ? np * (F)((c.BK / kin) * ((c.BM + 127) / 128)) : F(1);
-  f.DA_w = c.tmem_a ? l * e * c.BM * c.BK : F(0);
-  f.DA_r = c.tmem_a ? np * e * c.BM * c.BK : F(0);
+  f.D_w = f.D + (c.tmem_a ? l * e * c.BM * c.BK : F(0));
+  f.D_r = f.D + (c.tmem_a ? np * e * c.BM * c.BK : F(0));
   // measured: strategy B's tcgen05.cp per 128-row x 32-byte A slice, each charged L_mma
   if (c.tmem_a && measured) f.n_instr += l * (F)(c.BK * (int)e / 32) * (F)((c.BM + 127) / 128);
-  const F T_tmem = (f.D + f.DA_r) * th.inv[10] + f.n_instr * th.v[9] + (f.D + f.DA_w) * th.inv[11];
+  const F T_tmem = f.D_r * th.inv[10] + f.n_instr * th.v[9] + f.D_w * th.inv[11];
   const F T_mgmt = measured ? F(0) : th.v[13] / f.Kt;
   f.S = g == 1 ? F(1) : th.v[14];
   f.invS = g == 1 ? F(1) : th.inv[14];
@@ -341,9 +341,9 @@ __device__ __forceinline__ void step_store_adjoint(const pm_cfg& c, const ThetaT
   // T_c = X + (D + D_A,r)/BW_rd + n_instr L_mma + (D + D_A,w)/BW_wr + L_mgmt/K_tiles
   gR -= g_c * f.X * f.invR;
   gS -= g_c * f.X * f.invS;
-  d[10] -= g_c * ((f.D + f.DA_r) * th.inv[10]) * th.inv[10];
+  d[10] -= g_c * (f.D_r * th.inv[10]) * th.inv[10];
   d[9] += g_c * f.n_instr;
-  d[11] -= g_c * ((f.D + f.DA_w) * th.inv[11]) * th.inv[11];
+  d[11] -= g_c * (f.D_w * th.inv[11]) * th.inv[11];
   if (!measured) d[13] += g_c / f.Kt;
 }
 
@@ -384,13 +384,14 @@ __device__ __forceinline__ void gemm_adjoint(const pm_cfg& c, const ThetaT<F>& t
 }
 
 // The records that the search space and the calibration table are made of take
-// a shorter way to the same values: GEMM records of TMEM strategy A under the
-// measured reading with BM, BN in {64, 128, 256}, BK in {32, 64, 128}, 2..6 stages
+// a shorter way to the same values: GEMM records under the measured reading with BM, BN in {64, 128, 256}, BK in {32, 64, 128}, 2..6 stages
 // and extents below 2^20, whose counts fit in 32 bits and whose extents are
 // divided by shifts.  What depends on (dtype, cta_group) or on the stages alone
 // is looked up in shared memory: kernel parameters indexed by a lane's own value
 // are read once per distinct value.  The floating-point operations are
-// gemm_forward's, in its order, so the results are the same bits.
+// gemm_forward's, in its order, so the results are the same bits.  Both TMEM
+// strategies take it: rows of strategy B scattered over a table (the calibration's)
+// would send nearly every warp both ways (10^6 mixed records: 19.6 us, now 9.6).
 struct SpaceTables {
   float4 rate[6];       // by 2 dtype + (cta_group - 1): 1 / (R S), l e, n_p, 1 / R
   uint4 conc[2];        // by cta_group - 1: the wave division d - 1, m, s1, s2
@@ -421,10 +422,37 @@ __device__ __forceinline__ bool space_tables(const Theta& th, int n_sm, SpaceTab
 __device__ __forceinline__ bool in_space(const pm_cfg& c) {
   const unsigned tile = (unsigned)(uint16_t)c.BM | (unsigned)(uint16_t)c.BN << 16, bk = (unsigned)(uint16_t)c.BK;
   // one bit of 64..256 in each half of `tile`, one of 32..128 in bk
-  return c.kind == PM_KIND_GEMM && c.tmem_a == 0 && (unsigned)(c.stages - 2) <= 4u &&
+  return c.kind == PM_KIND_GEMM && (unsigned)c.tmem_a <= 1u && (unsigned)(c.stages - 2) <= 4u &&
          (unsigned)(c.cta_group - 1) <= 1u && (unsigned)c.dtype <= 2u && (tile & ~0x01C001C0u) == 0u &&
          (tile & 0xFFFFu) != 0u && (tile >> 16) != 0u && (tile & (tile - 0x00010001u)) == 0u && (bk & ~0xE0u) == 0u &&
          bk != 0u && (bk & (bk - 1u)) == 0u && ((unsigned)(c.M - 1) | (unsigned)(c.N - 1) | (unsigned)(c.K - 1)) < (1u << 20);
+}
+
+// The whole numbers of a record of the space: tensor-pipe instructions of a
+// K-step, bytes through TMEM (below 2^24), and whether the launch keeps one
+// accumulator buffer (single_buffer).
+struct SpaceInts {
+  int n_instr, d_r, d_w;
+  bool single;
+};
+
+__device__ __forceinline__ SpaceInts space_ints(const pm_cfg& c) {
+  SpaceInts r;
+  const int BM = c.BM, BN = c.BN, BK = c.BK, dt = c.dtype, blocks = 1 + (BM >> 8);
+  const int passes = dt == PM_FP32 ? 3 : 1, esh = 2 - dt;        // element bytes 4, 2, 1
+  r.n_instr = passes * (BK >> (3 + dt)) * blocks;
+  r.d_r = r.d_w = 4 * BM * BN;
+  if (c.tmem_a) {
+    const int a = BM * BK << esh, loads = dt == PM_FP32 ? 2 : 1;
+    r.d_r += passes * a;
+    r.d_w += loads * a;
+    r.n_instr += loads * ((BK << esh) >> 5) * blocks;
+    const int acc = (BM < 128 && c.cta_group == 2) ? BN >> 1 : blocks * BN;
+    r.single = 2 * acc + c.stages * blocks * (loads * (BK << esh) >> 2) > 512;
+  } else {
+    r.single = BM == 256 && BN == 256;                           // 512 columns
+  }
+  return r;
 }
 
 __device__ __forceinline__ void gemm_forward_space(const pm_cfg& c, const Theta& th, const SpaceTables& tab, GemmFwd& f) {
@@ -444,10 +472,11 @@ __device__ __forceinline__ void gemm_forward_space(const pm_cfg& c, const Theta&
   f.waves = (float)(int)((q + ((x - q) >> nc.z)) >> nc.w);
   f.Kt = (float)(int)((unsigned)(c.K + BK - 1) >> (5 + kb));
   f.D = (float)(4 * BM * BN);
-  const int blocks = 1 + (BM >> 8);
-  f.n_instr = np * (float)((BK >> (3 + c.dtype)) * blocks);
-  f.DA_w = f.DA_r = 0.f;
-  const float T_tmem = f.D * th.inv[10] + f.n_instr * th.v[9] + f.D * th.inv[11];
+  const SpaceInts si = space_ints(c);
+  f.n_instr = (float)si.n_instr;
+  f.D_r = (float)si.d_r;
+  f.D_w = (float)si.d_w;
+  const float T_tmem = f.D_r * th.inv[10] + f.n_instr * th.v[9] + f.D_w * th.inv[11];
   const int rows = gi == 0 ? max(BM, 128) : BM;
   f.X = (np * (float)(2 * rows * BN * BK)) * inv_rs;
   f.T_c = f.X + T_tmem;
@@ -468,7 +497,7 @@ __device__ __forceinline__ void gemm_forward_space(const pm_cfg& c, const Theta&
   f.ring = f.T_ring > f.T_eq8;
   f.T_step = f.ring ? f.T_ring : f.T_eq8;
   f.store_bytes = f.D;
-  f.drain = BM == 256 && BN == 256;                              // 512 columns: one accumulator buffer
+  f.drain = si.single;
   f.T_store = th.v[4] + f.store_bytes * th.inv[5] + (f.drain ? f.store_bytes * th.inv[17] : 0.f);
   f.launch = th.v[0] + th.v[13];
   f.T_stage = f.launch + f.waves * (f.Kt * f.T_step + f.T_store);
@@ -570,9 +599,9 @@ __device__ __forceinline__ pm_cfg load_cfg(const pm_cfg* p) {
   return c;
 }
 
-// Bound: ALU issue (210 warp-instructions per 32 configurations in the search
-// space, 377 for any others; 28 bytes each).  10^6 configurations 13.2 -> 8.5 us,
-// 10^7 114 -> 66 us with the short way of gemm_forward_space.  Six blocks per SM
+// Bound: ALU issue (about 215 warp-instructions per 32 configurations in the search
+// space, 377 for any others; 28 bytes each).  10^6 configurations 13.2 -> 8.9 us,
+// 10^7 114 -> 69 us with the short way of gemm_forward_space.  Six blocks per SM
 // (40 registers, no spills): 48 warps hide the latency of the dependent FP32
 // chain better than 40 or, at 32 registers, 64 (10^6: 11.0 us).
 __global__ void __launch_bounds__(256, 6) model_predict_kernel(const pm_cfg* __restrict__ cfgs, int64_t n, Theta th,
@@ -652,7 +681,7 @@ template <class F>
 constexpr int grad_min_blocks() { return sizeof(F) == 4 ? 4 : 2; }
 
 // Bound: FP32 ALU issue (10^6 configurations 25.1 -> 22.2 us with the sums by
-// halving, 14.8 us with the short way of gemm_forward_space; 10^7 218 -> 130 us);
+// halving, 15.3 us with the short way of gemm_forward_space; 10^7 218 -> 133 us);
 // FP64 at a calibration table's size the latency of one
 // configuration (1,901: 26.8 -> 12.8 us), at 10^6 the FP64 pipe (463 us).
 //
@@ -1356,8 +1385,8 @@ extern "C" pm_status pm_model_predict(const pm_cfg* cfgs_dev, int64_t n, const p
   PM_REQUIRE(cfgs_dev && theta_host && t_out_dev && n_sm > 0, PM_EINVAL, "null pointer or n_sm <= 0");
   PM_REQUIRE(((uintptr_t)cfgs_dev & 7) == 0, PM_EINVAL, "cfgs_dev must be 8-byte aligned");
   const int64_t want = (n + 255) / 256;
-  // one resident wave that walks the records up to eight rounds (10^6 records 8.5 us,
-  // 9.2 with 16 blocks per SM); past that smaller shares even out the SMs' speeds
+  // one resident wave that walks the records up to eight rounds (10^6 records 8.9 us,
+  // 9.6 with 16 blocks per SM); past that smaller shares even out the SMs' speeds
   // (10^7: 72 against 66 us)
   const int64_t resident = (int64_t)std::max(1, sm_count()) * 6;
   const int64_t cap = want <= 8 * resident ? resident : (int64_t)std::max(1, sm_count()) * 16;
