@@ -12,6 +12,7 @@
 #include <algorithm>
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "pm_internal.cuh"
@@ -508,6 +509,132 @@ __device__ __forceinline__ void gemm_forward_space(const pm_cfg& c, const Theta&
   f.T = f.T_stage >= f.T_rl ? f.T_stage : f.T_rl;
 }
 
+// The same way in FP64, with its adjoint.  An FP64 warp instruction holds its
+// scheduler's FP64 unit for 64 cycles on this GPU whatever its active lanes, so
+// what counts is their number: whole numbers stay integers (products up to 2^52
+// enter FP64 with one subtraction, the small ones through the bits of their exact
+// FP32 value with none), what depends on the parameters alone comes from the host,
+// and the one division by rho is a reciprocal used three times.  About 90
+// instructions for the prediction and its slopes in place of 200.
+template <class F>
+struct SpaceHost {};
+template <>
+struct SpaceHost<double> {
+  double inv_rs[6], inv_rsn[6], inv_r[6];    // by 2 dtype + (cta_group - 1): 1 / (R S), 1 / (n_SM R S), 1 / R
+  double oma[8], inv_s[8], inv_s1[8];        // by stages: 1 - alpha, 1 / s, and 1 / (s - 1) where alpha is free, else 0
+  double rho_m1, c3, ni10, ni11, t_sync, launch;   // rho_L2 - 1, its share of w0's slope, -1/BW^2, 2 L_mbar, launch
+  uint4 conc[2];                             // as SpaceTables
+  int ok;                                    // the launch's parameters allow the short way
+};
+
+static SpaceHost<double> make_space(const ThetaT<double>& th, int n_sm) {
+  SpaceHost<double> k = {};
+  for (int i = 0; i < 6; ++i) {
+    k.inv_r[i] = th.inv[6 + i / 2];
+    k.inv_rs[i] = k.inv_r[i] * (i % 2 ? th.inv[14] : 1.0);
+    k.inv_rsn[i] = k.inv_rs[i] * th.inv_nsm;
+  }
+  for (int s = 0; s < 8; ++s) {
+    const double r = th.v[15] * th.inv_s1[s];
+    k.oma[s] = r <= 0.0 ? 0.0 : (r >= 1.0 ? 1.0 : r);
+    k.inv_s[s] = th.inv_s[s];
+    k.inv_s1[s] = r > 0.0 && r < 1.0 ? th.inv_s1[s] : 0.0;
+  }
+  k.rho_m1 = th.v[16] - 1.0;
+  k.c3 = k.rho_m1 * th.inv[3] * th.inv[3];
+  k.ni10 = -(th.inv[10] * th.inv[10]);
+  k.ni11 = -(th.inv[11] * th.inv[11]);
+  k.t_sync = 2.0 * th.v[12];
+  k.launch = th.v[0] + th.v[13];
+  for (int i = 0; i < 2; ++i)
+    k.conc[i] = make_uint4(th.nc[i].d - 1u, th.nc[i].m, (unsigned)th.nc[i].s1, (unsigned)th.nc[i].s2);
+  k.ok = th.reading == PM_READING_MEASURED && th.nc_nsm == n_sm && th.v[3] > 0.0;
+  return k;
+}
+static SpaceHost<float> make_space(const ThetaT<float>&, int) { return {}; }
+
+// A positive integer that FP32 holds exactly, through FP32's bits.
+__device__ __forceinline__ double small_f64(int v) {
+  const unsigned b = __float_as_uint((float)v);
+  return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+// An integer in [0, 2^52): the low bits of 2^52 + v.
+__device__ __forceinline__ double large_f64(long long v) {
+  return __longlong_as_double(0x4330000000000000ll | v) - 4503599627370496.0;
+}
+
+// T_hat of a record of the space; its slopes are written to d (all NP entries).
+__device__ __forceinline__ double space_row(const pm_cfg& c, const ThetaT<double>& th, const SpaceHost<double>& k,
+                                            double (&d)[NP]) {
+  const int dt = c.dtype, gi = c.cta_group - 1, BM = c.BM, BN = c.BN, BK = c.BK, idx = 2 * dt + gi, s = c.stages;
+  const int passes = dt == PM_FP32 ? 3 : 1, le = dt == PM_FP32 ? 8 : 2 >> (dt - 1);
+  const SpaceInts si = space_ints(c);
+  const long long mn = (long long)c.M * c.N;
+  const double W = large_f64(le * ((long long)(c.M + c.N) * c.K) + 4 * mn);
+  const unsigned tm = (unsigned)(c.M + (BM << gi) - 1) >> (6 + (BM >> 7) + gi);
+  const unsigned tn = (unsigned)(c.N + BN - 1) >> (6 + (BN >> 7));
+  const uint4 nc = k.conc[gi];
+  const unsigned x = ((tm * tn) << gi) + nc.x, q = __umulhi(nc.y, x);
+  const double waves = large_f64((long long)((q + ((x - q) >> nc.z)) >> nc.w));
+  const double Kt = small_f64((int)((unsigned)(c.K + BK - 1) >> (5 + (BK >> 6))));
+  const double D = small_f64(4 * BM * BN), D_r = small_f64(si.d_r), D_w = small_f64(si.d_w), n_i = small_f64(si.n_instr);
+  const double inv_rs = k.inv_rs[idx], inv_s = k.inv_s[s], oma = k.oma[s];
+  const double X = small_f64(passes * 2 * (gi == 0 ? max(BM, 128) : BM) * BN * BK) * inv_rs;
+  const double E = exp(-W * th.inv[3]);
+  const double inv_rho = __drcp_rn(fma(k.rho_m1, E, 1.0));
+  const double t_bw = small_f64(le * BK * (BM + (BN >> gi))) * th.inv[5] * inv_rho;
+  const double T_tma = th.v[4] + t_bw;
+  const double T_c = X + fma(D_w, th.inv[11], fma(n_i, th.v[9], D_r * th.inv[10]));
+  const double T_io = oma * T_tma;
+  const bool c_first = T_c >= T_io;
+  const double T_eq8 = fmax(T_c, T_io) + k.t_sync;
+  const double T_ring = (T_tma + T_c + k.t_sync) * inv_s;
+  const bool ring = T_ring > T_eq8;
+  const double d5 = D * th.inv[5];
+  double T_store = th.v[4] + d5, d17 = 0.0;
+  if (si.single) {
+    d17 = D * th.inv[17];
+    T_store += d17;
+  }
+  const double T_stage = fma(waves, fma(Kt, ring ? T_ring : T_eq8, T_store), k.launch);
+  const double A_rl = large_f64(2 * passes * mn) * small_f64(c.K) * k.inv_rsn[idx], B_rl = W * th.inv[2];
+  const bool a_first = A_rl >= B_rl;
+  const double T_rl = k.launch + (a_first ? A_rl : B_rl);
+  const bool stage = T_stage >= T_rl;
+  // slopes (step_store_adjoint, gemm_adjoint): the roofline branch has no share
+  // in the tiles' terms
+  const double g_w = stage ? waves : 0.0, g_step = g_w * Kt, g_ring = g_step * inv_s;
+  const double g_c = ring ? g_ring : (c_first ? g_step : 0.0), g_io = ring || c_first ? 0.0 : g_step;
+  const double g_tma = ring ? g_ring : g_io * oma, g_bw = g_tma * t_bw, g_E = -(g_bw * inv_rho) * E, g_x = g_c * X;
+  double g_R = -(g_x * k.inv_r[idx]), g_S = gi ? -(g_x * th.inv[14]) : 0.0;
+  d[2] = 0.0;
+  if (!stage) {
+    if (a_first) {
+      g_R = -(A_rl * k.inv_r[idx]);
+      g_S = gi ? -(A_rl * th.inv[14]) : 0.0;
+    } else {
+      d[2] = -(B_rl * th.inv[2]);
+    }
+  }
+  d[0] = d[13] = 1.0;
+  d[1] = 0.0;
+  d[3] = g_E * W * k.c3;
+  d[4] = g_w + g_tma;
+  d[5] = -(fma(g_w, d5, g_bw) * th.inv[5]);
+  d[6] = dt == PM_FP32 ? g_R : 0.0;
+  d[7] = dt == PM_BF16 ? g_R : 0.0;
+  d[8] = dt == PM_FP8E4M3 ? g_R : 0.0;
+  d[9] = g_c * n_i;
+  d[10] = g_c * D_r * k.ni10;
+  d[11] = g_c * D_w * k.ni11;
+  d[12] = 2.0 * (ring ? g_ring : g_step);
+  d[14] = g_S;
+  d[15] = g_io * T_tma * k.inv_s1[s];
+  d[16] = g_E;
+  d[17] = si.single ? -(g_w * d17 * th.inv[17]) : 0.0;
+  return stage ? T_stage : T_rl;
+}
+
 // Memory probes.  Copy/triad through Eq. 16 with W = beta bytes moved;
 // TMA2D: tile latency plus ceil(tiles/SMs) tile round trips (Eq. 4),
 // bounded below by the streaming time of Eq. 16.
@@ -575,6 +702,52 @@ __device__ __forceinline__ void probe_adjoint(const pm_cfg& c, const ThetaT<F>& 
       bw_adjoint(th, f, -w * f.beta / (f.Bw * f.Bw), d);
     }
   }
+}
+
+// probe_forward and probe_adjoint in FP64 with one reciprocal in place of five
+// divisions, the three kinds in step: a calibration table's few probe rows share a
+// warp with its last GEMM rows, and the slowest warp ends the kernel (1,901 mixed
+// records 13.0 -> 11.5 us).
+__device__ __forceinline__ double probe_row(const pm_cfg& c, const ThetaT<double>& th, int n_sm, double (&d)[NP]) {
+  const bool tma = c.kind == PM_KIND_TMA2D;
+  double beta, other;                            // bytes, and the time that Eq. 16 is weighed against
+  double other_slope;
+  if (tma) {
+    const int64_t nt = cdiv(c.M, c.BM) * cdiv(c.N, c.BN);
+    beta = 8.0 * c.M * c.N;
+    other_slope = (double)cdiv(nt, n_sm) * (8.0 * c.BM * c.BN) * th.inv[5];
+    other = th.v[4] + other_slope;
+  } else {
+    beta = (c.kind == PM_KIND_COPY ? 8.0 : 12.0) * c.M;
+    other_slope = other = beta * th.inv[2];
+  }
+  const bool blend = th.v[3] > 0.0;
+  const double x = beta * th.inv[3], E = blend ? exp(-x) : 0.0, dB = th.v[2] - th.v[1];
+  const double inv_bw = __drcp_rn(blend ? fma(dB, E, th.v[1]) : th.v[1]);
+  const double stream = beta * inv_bw;
+  // ties go to the first argument: the stream's time of copy and triad, the tiles' of TMA
+  const double T_s = th.v[0] + stream, T_o = th.v[0] + other;
+  const bool by_stream = tma ? !(T_o >= T_s) : T_s >= T_o;
+#pragma unroll
+  for (int j = 0; j < NP; ++j) d[j] = 0.0;
+  d[0] = 1.0;
+  if (by_stream) {
+    const double gB = -(stream * inv_bw);
+    if (blend) {
+      const double gE = gB * E;
+      d[1] = gB - gE;
+      d[2] = gE;
+      d[3] = gE * dB * x * th.inv[3];
+    } else {
+      d[1] = gB;
+    }
+  } else if (tma) {
+    d[4] = 1.0;
+    d[5] = -(other_slope * th.inv[5]);
+  } else {
+    d[2] = -(other_slope * th.inv[2]);
+  }
+  return by_stream ? T_s : T_o;
 }
 
 // A record the model can evaluate on n_sm SMs; a CTA pair (cta_group 2)
@@ -682,8 +855,8 @@ constexpr int grad_min_blocks() { return sizeof(F) == 4 ? 4 : 2; }
 
 // Bound: FP32 ALU issue (10^6 configurations 25.1 -> 22.2 us with the sums by
 // halving, 15.3 us with the short way of gemm_forward_space; 10^7 218 -> 133 us);
-// FP64 at a calibration table's size the latency of one
-// configuration (1,901: 26.8 -> 12.8 us), at 10^6 the FP64 pipe (463 us).
+// FP64 at every size the FP64 units (1,901 configurations 26.8 -> 12.8 us on
+// clusters, 10.3 with space_row; 10^6 486 -> 312 us).
 //
 // One partial record per kGradThreads threads, the threads of a record spread
 // over a cluster of CL blocks: partials[j * records + r] is component j of
@@ -691,21 +864,31 @@ constexpr int grad_min_blocks() { return sizeof(F) == 4 ? 4 : 2; }
 // the sums are the same, term by term, whatever CL.
 template <class F, int CL>
 __global__ void __launch_bounds__(kGradThreads / CL, CL == 1 ? grad_min_blocks<F>() : 1)
-    model_grad_kernel(const pm_cfg* __restrict__ cfgs, int64_t n, const __grid_constant__ ThetaT<F> th, int n_sm,
-                      const F* __restrict__ t_meas, double* __restrict__ partials) {
+    model_grad_kernel(const pm_cfg* __restrict__ cfgs, int64_t n, const __grid_constant__ ThetaT<F> th,
+                      const __grid_constant__ SpaceHost<F> sh, int n_sm, const F* __restrict__ t_meas,
+                      double* __restrict__ partials) {
   constexpr int kThreads = kGradThreads / CL;
   grid_dependents_launch();                      // the finish kernel may be set up (it waits for this grid)
   if constexpr (CL > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   const int records = (int)(gridDim.x / CL), rec = (int)(blockIdx.x / CL), part = (int)(blockIdx.x % CL);
-  __shared__ SpaceTables tab;
-  bool space = false;
-  if constexpr (sizeof(F) == 4) space = space_tables(th, n_sm, tab);
+  // the short way's tables, in shared memory (lanes index them by their own record)
+  __shared__ std::conditional_t<sizeof(F) == 4, SpaceTables, SpaceHost<F>> tab;
+  bool space;
+  if constexpr (sizeof(F) == 4) {
+    space = space_tables(th, n_sm, tab);
+  } else {
+    const int* from = reinterpret_cast<const int*>(&sh);
+    for (int w = threadIdx.x; w < (int)(sizeof(sh) / 4); w += kThreads) reinterpret_cast<int*>(&tab)[w] = from[w];
+    __syncthreads();
+    space = sh.ok != 0;
+  }
   F acc[NREC];                                   // loss, then the gradient
 #pragma unroll
   for (int j = 0; j < NREC; ++j) acc[j] = F(0);
   for (int64_t i = (int64_t)rec * kGradThreads + part * kThreads + threadIdx.x; i < n;
        i += (int64_t)records * kGradThreads) {
     const pm_cfg c = load_cfg(cfgs + i);
+    const F log_t = pm_log(__ldg(t_meas + i));
     F d[NP];
 #pragma unroll
     for (int j = 0; j < NP; ++j) d[j] = F(0);
@@ -716,6 +899,8 @@ __global__ void __launch_bounds__(kGradThreads / CL, CL == 1 ? grad_min_blocks<F
         gemm_forward_space(c, th, tab, f);
         T = f.T;
         gemm_adjoint<true>(c, th, f, F(1), d);
+      } else {
+        T = space_row(c, th, tab, d);
       }
     } else if (!cfg_sane(c, n_sm)) {
       T = (F)__int_as_float(0x7fc00000);
@@ -724,13 +909,15 @@ __global__ void __launch_bounds__(kGradThreads / CL, CL == 1 ? grad_min_blocks<F
       gemm_forward(c, th, n_sm, f);
       T = f.T;
       gemm_adjoint(c, th, f, F(1), d);
-    } else {
+    } else if constexpr (sizeof(F) == 4) {
       ProbeFwdT<F> f;
       probe_forward(c, th, n_sm, f);
       T = f.T;
       probe_adjoint(c, th, f, F(1), d);
+    } else {
+      T = probe_row(c, th, n_sm, d);
     }
-    const F r = pm_log(T) - pm_log(__ldg(t_meas + i));
+    const F r = pm_log(T) - log_t;
     acc[0] = fma(r, r, acc[0]);
     const F w = F(2) * r / T;
 #pragma unroll
@@ -1408,10 +1595,12 @@ template <class F>
 static pm_status launch_grad(const pm_cfg* cfgs, int64_t n, const ThetaT<F>& th, int n_sm, const F* t_meas,
                              double* partials, int records, double* out, cudaStream_t s) {
   // FP64, few records: a cluster of eight one-warp blocks per record.  Measured
-  // with / without clusters: 1,901 configurations 12.8 / 21.0 us, 20,000 15.9 / 21.3,
-  // 30,000 19.6 / 21.4, 38,000 33.2 / 21.5 (the clusters no longer fit at once).  The
+  // with / without clusters, before space_row: 1,901 configurations 12.8 / 21.0 us,
+  // 20,000 15.9 / 21.3, 30,000 19.6 / 21.4, 38,000 33.2 / 21.5 (the clusters no longer
+  // fit at once).  The
   // FP32 kernel is bound by one thread's latency and gains nothing.
   constexpr int CL = sizeof(F) == 8 ? 8 : 1;
+  const SpaceHost<F> sh = make_space(th, n_sm);
   cudaLaunchConfig_t cfg = {};
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -1424,10 +1613,10 @@ static pm_status launch_grad(const pm_cfg* cfgs, int64_t n, const ThetaT<F>& th,
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, model_grad_kernel<F, CL>, cfgs, n, th, n_sm, t_meas, partials);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, model_grad_kernel<F, CL>, cfgs, n, th, sh, n_sm, t_meas, partials);
     if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchKernelEx(model_grad_kernel)");
   } else {
-    model_grad_kernel<F, 1><<<records, kGradThreads, 0, s>>>(cfgs, n, th, n_sm, t_meas, partials);
+    model_grad_kernel<F, 1><<<records, kGradThreads, 0, s>>>(cfgs, n, th, sh, n_sm, t_meas, partials);
     pm_status st = launch_status("model_grad_kernel");
     if (st != PM_OK) return st;
   }

@@ -202,3 +202,28 @@ def test_short_way_agrees_with_the_general_one(lib, reading):
         wrong = np.ones(n, bool) if f in ("M", "kind") else c["kind"] == 0
         assert np.all(np.isnan(t.cpu().numpy()[wrong])), f
         bad[f][:] = c[f]
+
+
+@pytest.mark.parametrize("n_sm", [152, 3])
+@pytest.mark.parametrize("w0", [None, 0.0])
+def test_fp64_short_ways_agree_with_oracle(lib, reading, n_sm, w0):
+    # every kind of record in one table; without the L2 blend the general way
+    n = 20000
+    c = edge_cfgs(n, 70)
+    probes = np.arange(n) >= n - 600
+    c["kind"][~probes] = 0
+    c["kind"][probes] = 1 + np.arange(600) // 200
+    th = O.prior_theta(N_SM, reading=reading)
+    if w0 is not None:
+        th[3] = w0
+    t_o, gi = O.model_batch(c, th, n_sm, grad=True)
+    t_meas = t_o * np.exp(0.3 * (S.uniform01_f64(71, n) - 0.5))
+    L_o, g_o = O.model_loss_grad(c, th, n_sm, t_meas)
+    r = np.log(t_o) - np.log(t_meas)
+    scale = (2.0 / n) * np.sum(np.abs(r[:, None] * gi / t_o[:, None]), axis=0)
+    ws = torch.empty(lib.pm_model_grad_workspace(n) // 8, dtype=torch.float64, device="cuda")
+    out = torch.empty(lib.N_GRAD_OUT, dtype=torch.float64, device="cuda")
+    lib.pm_model_grad_f64(lib.cfg_tensor(c), n, th, n_sm, torch.from_numpy(t_meas).cuda(), ws, out)
+    o = out.cpu().numpy()
+    assert o[0] == pytest.approx(L_o, rel=1e-10)
+    assert np.all(np.abs(o[1:] - g_o) <= 1e-10 * scale + 1e-300)
