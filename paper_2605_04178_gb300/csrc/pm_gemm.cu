@@ -1047,13 +1047,19 @@ extern "C" pm_status pm_gemm_autotune(const pm_cfg* shape, int32_t k, const pm_p
 // copied and converted first, then A moves in row chunks on a copy stream,
 // each chunk is converted and multiplied on a compute stream while the next
 // chunk is in flight, and each finished C chunk returns on a third stream.
-// Two staging buffers per chunked operand; events order reuse.
+// Two staging buffers per chunked operand; events order reuse.  The chunks of
+// either buffer have their own compute stream: a chunk's product has few tiles
+// and is bound by its K-loop's latency (44 us for 512 x 4096 x 4096, on 32 SMs),
+// so one after another they, not the host link, set the pace.  BF16 4096^3 in 8 / 16 /
+// 32 chunks 907 / 1250 / 1950 -> 890 / 1036 / 1448 us (floor 640: both inputs over the
+// link), FP32 1024^3 in 4 / 8 chunks 170 / 266 -> 125 / 178.  At 8 chunks the result's
+// way back beside the inputs (155 against 195 GB/s alone) is the longest chain.
 namespace pm {
 
 struct HostPipe {
   int dev = -1;
-  cudaStream_t s_in = nullptr, s_comp = nullptr, s_out = nullptr;
-  cudaEvent_t start, b_ready, done, a_loaded[2], a_free[2], c_ready[2], c_free[2];
+  cudaStream_t s_in = nullptr, s_comp[2] = {nullptr, nullptr}, s_out = nullptr;
+  cudaEvent_t start, b_ready, b_op, done, a_loaded[2], a_free[2], c_ready[2], c_free[2];
 };
 static thread_local HostPipe g_pipe;
 
@@ -1063,11 +1069,12 @@ void release_host_pipe_this_thread() {
   int cur = -1;
   cudaGetDevice(&cur);
   if (cudaSetDevice(P.dev) == cudaSuccess) {
-    cudaEvent_t evs[] = {P.start, P.b_ready, P.done, P.a_loaded[0], P.a_loaded[1], P.a_free[0],
+    cudaEvent_t evs[] = {P.start, P.b_ready, P.b_op, P.done, P.a_loaded[0], P.a_loaded[1], P.a_free[0],
                          P.a_free[1], P.c_ready[0], P.c_ready[1], P.c_free[0], P.c_free[1]};
     for (cudaEvent_t e : evs) cudaEventDestroy(e);
     cudaStreamDestroy(P.s_in);
-    cudaStreamDestroy(P.s_comp);
+    cudaStreamDestroy(P.s_comp[0]);
+    cudaStreamDestroy(P.s_comp[1]);
     cudaStreamDestroy(P.s_out);
   }
   P = HostPipe();
@@ -1081,9 +1088,9 @@ static pm_status host_pipe() {
   if (P.dev == dev) return PM_OK;
   PM_REQUIRE(P.dev < 0, PM_EUNSUPPORTED, "pm_gemm_host: one device per host thread");
   PM_CUDA(cudaStreamCreateWithFlags(&P.s_in, cudaStreamNonBlocking));
-  PM_CUDA(cudaStreamCreateWithFlags(&P.s_comp, cudaStreamNonBlocking));
+  for (cudaStream_t& s : P.s_comp) PM_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
   PM_CUDA(cudaStreamCreateWithFlags(&P.s_out, cudaStreamNonBlocking));
-  cudaEvent_t* evs[] = {&P.start, &P.b_ready, &P.done, &P.a_loaded[0], &P.a_loaded[1], &P.a_free[0],
+  cudaEvent_t* evs[] = {&P.start, &P.b_ready, &P.b_op, &P.done, &P.a_loaded[0], &P.a_loaded[1], &P.a_free[0],
                         &P.a_free[1], &P.c_ready[0], &P.c_ready[1], &P.c_free[0], &P.c_free[1]};
   for (cudaEvent_t* e : evs) PM_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
   P.dev = dev;
@@ -1155,19 +1162,22 @@ extern "C" pm_status pm_gemm_host(const pm_cfg* cfg, const float* A_host, const 
   PM_REQUIRE((K + 31) / 32 <= 65535, PM_EINVAL, "K too large for the transpose grid");
   PM_CUDA(cudaEventRecord(P.start, caller));
   PM_CUDA(cudaStreamWaitEvent(P.s_in, P.start, 0));
-  PM_CUDA(cudaStreamWaitEvent(P.s_comp, P.start, 0));
+  for (cudaStream_t sc : P.s_comp) PM_CUDA(cudaStreamWaitEvent(sc, P.start, 0));
   PM_CUDA(cudaStreamWaitEvent(P.s_out, P.start, 0));
   // B: copy, then convert to the K-major operand
   PM_CUDA(cudaMemcpyAsync(b32, B_host, (size_t)K * N * 4, cudaMemcpyHostToDevice, P.s_in));
   PM_CUDA(cudaEventRecord(P.b_ready, P.s_in));
-  PM_CUDA(cudaStreamWaitEvent(P.s_comp, P.b_ready, 0));
-  if (dt == PM_FP8E4M3) PM_CUDA(cudaMemsetAsync(scales + 2, 0, 2 * sizeof(unsigned int), P.s_comp));
-  st = launch_prepare(dt, nullptr, 0, b32, K, N, nullptr, bop, scales, P.s_comp);
+  PM_CUDA(cudaStreamWaitEvent(P.s_comp[0], P.b_ready, 0));
+  if (dt == PM_FP8E4M3) PM_CUDA(cudaMemsetAsync(scales + 2, 0, 2 * sizeof(unsigned int), P.s_comp[0]));
+  st = launch_prepare(dt, nullptr, 0, b32, K, N, nullptr, bop, scales, P.s_comp[0]);
   if (st != PM_OK) return st;
+  PM_CUDA(cudaEventRecord(P.b_op, P.s_comp[0]));
+  PM_CUDA(cudaStreamWaitEvent(P.s_comp[1], P.b_op, 0));
   // A in row chunks
   const int nch = (int)((M + Lh.Mc - 1) / Lh.Mc);
   for (int i = 0; i < nch; ++i) {
     const int j = i & 1;
+    const cudaStream_t sc = P.s_comp[j];
     const int64_t r0 = (int64_t)i * Lh.Mc;
     const int rows = (int)std::min<int64_t>(Lh.Mc, M - r0);
     float* a32 = reinterpret_cast<float*>(ws + Lh.off_a32[j]);
@@ -1176,16 +1186,16 @@ extern "C" pm_status pm_gemm_host(const pm_cfg* cfg, const float* A_host, const 
     if (i >= 2) PM_CUDA(cudaStreamWaitEvent(P.s_in, P.a_free[j], 0));
     PM_CUDA(cudaMemcpyAsync(a32, A_host + r0 * K, (size_t)rows * K * 4, cudaMemcpyHostToDevice, P.s_in));
     PM_CUDA(cudaEventRecord(P.a_loaded[j], P.s_in));
-    PM_CUDA(cudaStreamWaitEvent(P.s_comp, P.a_loaded[j], 0));
-    st = launch_prepare(dt, a32, rows, nullptr, K, N, aop, nullptr, scales, P.s_comp);
+    PM_CUDA(cudaStreamWaitEvent(sc, P.a_loaded[j], 0));
+    st = launch_prepare(dt, a32, rows, nullptr, K, N, aop, nullptr, scales, sc);
     if (st != PM_OK) return st;
-    PM_CUDA(cudaEventRecord(P.a_free[j], P.s_comp));
-    if (i >= 2) PM_CUDA(cudaStreamWaitEvent(P.s_comp, P.c_free[j], 0));
+    PM_CUDA(cudaEventRecord(P.a_free[j], sc));
+    if (i >= 2) PM_CUDA(cudaStreamWaitEvent(sc, P.c_free[j], 0));
     pm_cfg cc = *cfg;
     cc.M = rows;
-    st = gemm_launch(cc, aop, bop, cd, scales, P.s_comp);
+    st = gemm_launch(cc, aop, bop, cd, scales, sc);
     if (st != PM_OK) return st;
-    PM_CUDA(cudaEventRecord(P.c_ready[j], P.s_comp));
+    PM_CUDA(cudaEventRecord(P.c_ready[j], sc));
     PM_CUDA(cudaStreamWaitEvent(P.s_out, P.c_ready[j], 0));
     PM_CUDA(cudaMemcpyAsync(C_host + r0 * N, cd, (size_t)rows * N * 4, cudaMemcpyDeviceToHost, P.s_out));
     PM_CUDA(cudaEventRecord(P.c_free[j], P.s_out));
