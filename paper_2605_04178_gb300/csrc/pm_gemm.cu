@@ -6,11 +6,10 @@
 //
 // Kernel shape (sm_103a): one persistent CTA per SM (CTA pair per two SMs for
 // cta_group 2), 6 warps:
-//   warp 0      TMA producer (one thread): waits empty[s], loads stage s;
-//   warp 1      TMEM allocator and MMA issuer: the whole warp runs the
-//               K-loop (waits full[s], forms the descriptors) and one lane
-//               issues BK/k_instr MMAs per row block and commits to
-//               empty[s]; after the last K-step it commits to acc_full[buffer];
+//   warp 0      TMA producer: waits empty[s], loads stage s;
+//   warp 1      TMEM allocator and MMA issuer: waits full[s], issues
+//               BK/k_instr MMAs per row block and commits to empty[s]; after
+//               the last K-step it commits to acc_full[buffer];
 //   warps 2..5  epilogue: wait acc_full, tcgen05.ld 32-column chunks, scale,
 //               store FP32 C (masked at the M/N edges), release the buffer.
 // TMEM strategy A keeps only the accumulators in tensor memory and feeds both
@@ -23,6 +22,18 @@
 // tile i+1 starts on row block 0 while the epilogue still drains row block 1.  Each CTA of a pair loads its own A
 // rows and half of B (traffic 2 M_A + M_B per pair, no multicast); the pair
 // leader issues the cta_group::2 MMAs.
+//
+// Warps 0 and 1 run their K-loops converged (waits, addresses and descriptors
+// in all lanes) and one elected lane issues, each instruction under its
+// predicate.  Where a tile has few MMA cycles a K-step, the step is bound by
+// these two instruction streams (some 300 cycles for the loads, 400 for the
+// MMAs), not by memory or the tensor core.  One producer thread, with the warp
+// index from threadIdx alone, against this form: BF16 64 x 4096 x 4096 (64x128
+// tiles) 25 -> 19 us, 20 x 8192 x 8192 (64x64) 41 -> 30.5, 1024^3 (128x128)
+// 9.3 -> 7.0, 8192^3 with 128x256 pair tiles 665 -> 637, FP32 512^3 13.1 ->
+// 12.4; 256x256 pair tiles (tensor-bound) the same.  Lane 0 in place of the
+// elected lane: 23.4, 34.4, 8.1, 641, 12.3.  The MMAs of a step in a branch of
+// the elected lane: 21, 32, 7.7, 640, 12.5.
 #include <stdlib.h>
 
 #include <algorithm>
@@ -307,7 +318,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 
   constexpr int L = (KIND == 1) ? 2 : 1;              // operand halves (hi, lo) for three-pass TF32
   constexpr int E = (KIND == 0) ? 2 : (KIND == 1 ? 4 : 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // the warp index through a shuffle, so that the compiler knows it to be the
+  // same in all lanes and keeps the roles' loops on the uniform datapath
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const uint32_t rank = (CG == 2) ? cluster_ctarank() : 0u;
   const int cta = (CG == 2) ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const int n_ctas = (CG == 2) ? (int)(gridDim.x >> 1) : (int)gridDim.x;
@@ -351,7 +364,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    // the whole warp runs the loop in step; one lane issues
+    {
+      const uint32_t issue = elect_one() ? 1u : 0u;
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
@@ -364,21 +379,23 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         const CUtensorMap* ma = &maps.a[T.ma];
         const CUtensorMap* mb = &maps.b[T.mb];
         for (int kt = 0; kt < p.Kt; ++kt) {
-          if (!mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1u, p.wd, abort_p, SITE_GEMM_PRODUCER)) {
+          if (!warp_wait(smem_u32(&empty_bar[stage]), phase ^ 1u, p.wd, abort_p, SITE_GEMM_PRODUCER)) {
             ok = false;
             break;
           }
           const uint32_t fb = smem_u32(&full_bar[stage]);
           uint32_t fbc = fb;
           if constexpr (CG == 1) {
-            mbar_arrive_expect_tx(fb, T.tx);
+            if (issue) mbar_arrive_expect_tx(fb, T.tx);
+            __syncwarp();
           } else {
             // The leader arms its own full barrier for both CTAs' bytes; the
             // peer only points its TMA completions at that barrier (a
             // completion that lands before the arming leaves the phase pending
             // until the leader's arrival).
             fbc = mapa_shared(fb, 0);
-            if (rank == 0) mbar_arrive_expect_tx(fb, 2u * T.tx);
+            if (rank == 0 && issue) mbar_arrive_expect_tx(fb, 2u * T.tx);
+            __syncwarp();
           }
           const uint32_t sbase = base + (uint32_t)stage * p.stage_bytes;
           const uint32_t bbase = sbase + (uint32_t)(L * p.n_atoms) * T.a_part;
@@ -389,11 +406,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
               const uint32_t da = sbase + (uint32_t)(h * p.n_atoms + a) * T.a_part;
               const uint32_t db = bbase + (uint32_t)(h * p.n_atoms + a) * T.b_part;
               if constexpr (CG == 1) {
-                tma_load_2d(da, ma, fb, x, T.arow + h * p.lo_row_a);
-                tma_load_2d(db, mb, fb, x, T.brow + h * p.lo_row_b);
+                tma_load_2d(da, ma, fb, x, T.arow + h * p.lo_row_a, issue);
+                tma_load_2d(db, mb, fb, x, T.brow + h * p.lo_row_b, issue);
               } else {
-                tma_load_2d_pair(da, ma, fbc, x, T.arow + h * p.lo_row_a);
-                tma_load_2d_pair(db, mb, fbc, x, T.brow + h * p.lo_row_b);
+                tma_load_2d_pair(da, ma, fbc, x, T.arow + h * p.lo_row_a, issue);
+                tma_load_2d_pair(db, mb, fbc, x, T.brow + h * p.lo_row_b, issue);
               }
             }
           }
@@ -403,9 +420,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------- MMA issuer
-    // the whole warp runs the loop in step; lane 0 issues
+    // the whole warp runs the loop in step; one lane issues
     if (rank == 0) {
-      MmaRing r{full_bar, empty_bar, acce_bar, 0, 0u, lane == 0 ? 1u : 0u};
+      MmaRing r{full_bar, empty_bar, acce_bar, 0, 0u, elect_one() ? 1u : 0u};
       bool ok = true;
       int it = 0;
       int qh = 0;
@@ -512,8 +529,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             // write along the rows of C, one 128-byte row segment per store (four
             // where rows are 16-byte multiples) instead of one element of 32
             // rows, which cost 32 requests a store and bound the kernel.  BF16
-            // 4096 x 4095 x 256 96 -> 30 us, 4096 x 4095 x 4096 181 -> 117, 1000 x 1003 x
-            // 1040 17.9 -> 11.2, FP8 300 x 2941 x 528 14.5 -> 8.2.  (Chunks whose rows
+            // 4096 x 4095 x 256 96 -> 30 us (22.5 with the roles in step), 4096 x 4095 x
+            // 4096 181 -> 117 (106), 1000 x 1003 x 1040 17.9 -> 11.2 (9.1), FP8 300 x 2941
+            // x 528 14.5 -> 8.2 (7.1).  (Chunks whose rows
             // allow 16-byte stores are left to the lanes beside TMA and in 64-row
             // tiles: staging them made the single-buffered 256 x 256 tiles of grouped
             // launches 2-3 % slower.)
@@ -676,7 +694,8 @@ pm_status cached_tmap(CUtensorMap* out, const void* ptr, int dtcode, uint64_t ro
 // The kernel is launched to overlap the end of the previous kernel of its stream
 // (programmatic dependent launch): its barriers, TMEM and tensor maps are set up
 // while that one's last blocks run.  Back to back, 1024^3 BF16 11.6-13 -> 9.1 us a launch,
-// FP32 512^3 14.7 -> 13.2, 4096 x 4096 x 256 20.7 -> 17.6, 4096^3 91.0 -> 89.2; of no account at 8192^3.
+// FP32 512^3 14.7 -> 13.2, 4096 x 4096 x 256 20.7 -> 17.6, 4096^3 91.0 -> 89.2; of no account at
+// 8192^3 (now, with the roles in step, 7.0, 12.3, 16.6 and 87.7).
 template <int CG, int KIND, int TA, int MAXG>
 static pm_status launch_gemm_table(const TensorMaps& maps, const GroupTableT<MAXG>& g, const GemmParams& p, int grid,
                                    size_t smem, cudaStream_t s) {
@@ -826,7 +845,7 @@ static pm_status plan_launch(int dt, int cg, int BK, int stages, int tmem_a, int
   P.smem = (size_t)stages * stage + 1024;
   // epilogue staging after the ring: two 4 KB buffers per warp (which TMA stores
   // need), or one where no more fits (256 x 64 x 64 BF16, 5 stages, 8000 x 8000 x 512:
-  // 152 -> 124 us, with 7999 columns 465 -> 139); without any, lanes store their rows
+  // 152 -> 124 us, now 115; with 7999 columns 465 -> 139, now 105); without any, lanes store their rows
   p.staging_off = (uint32_t)stages * stage;
   p.tma_store = 0;
   p.c_rows = (int)sum_m;
