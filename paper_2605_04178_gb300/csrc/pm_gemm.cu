@@ -174,12 +174,11 @@ __device__ __forceinline__ constexpr uint32_t ta_col(int h, int a, int kk, int m
 // NK = swizzle span / 32 B k-steps per atom, NMBLK 128-row blocks; three-pass
 // TF32 adds the hi.lo and lo.hi products.  TA (strategy B): the stage's A
 // slices are first copied to TMEM at a_tm and the MMAs read A from there.
-template <int CG, int KIND, int NATOMS, int NK, int NMBLK, int TA>
+template <int CG, int KIND, int NATOMS, int NK, int NMBLK, int TA, int P0 = 0, int P1 = (KIND == 1 ? 3 : 1)>
 __device__ __forceinline__ void issue_stage(uint32_t d0, uint64_t a0, uint64_t b0, uint32_t a_part16,
                                             uint32_t b_part16, uint32_t mblk16, uint32_t idesc, uint32_t bn,
                                             bool first, uint32_t a_tm, uint32_t issue) {
-  constexpr int PASSES = (KIND == 1) ? 3 : 1;
-  if constexpr (TA) {
+  if constexpr (TA && P0 == 0) {
     constexpr int L = (KIND == 1) ? 2 : 1;
 #pragma unroll
     for (int h = 0; h < L; ++h)
@@ -193,7 +192,7 @@ __device__ __forceinline__ void issue_stage(uint32_t d0, uint64_t a0, uint64_t b
                              a0 + (uint64_t)((h * NATOMS + a) * a_part16 + m * mblk16 + 2u * kk), issue);
   }
 #pragma unroll
-  for (int pass = 0; pass < PASSES; ++pass) {
+  for (int pass = P0; pass < P1; ++pass) {
     const uint32_t ha = (pass == 2) ? 1u : 0u, hb = (pass == 1) ? 1u : 0u;
 #pragma unroll
     for (int a = 0; a < NATOMS; ++a) {
@@ -219,6 +218,7 @@ __device__ __forceinline__ void issue_stage(uint32_t d0, uint64_t a0, uint64_t b
 // Barriers and buffers the MMA issuer's K-loop works with.
 struct MmaRing {
   uint64_t* full;
+  uint64_t* full_lo;               // three-pass TF32: the stage's low planes
   uint64_t* empty;
   uint64_t* acce;
   int stage;
@@ -233,15 +233,24 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, const W
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, wd, abort_p, site)) != 0;
 }
 
-// One K-step's MMAs and the commit that frees its ring stage.
-template <int CG, int KIND, int NA, int NK, int NM, int TA>
-__device__ __forceinline__ void mma_step(MmaRing& r, const GemmParams& p, uint32_t d0, uint64_t a0, uint64_t b0,
+// One K-step's MMAs and the commit that frees its ring stage.  LO: the low planes
+// have a barrier of their own, waited for after the pass over the high ones.
+template <int CG, int KIND, int NA, int NK, int NM, int TA, int LO>
+__device__ __forceinline__ bool mma_step(MmaRing& r, const GemmParams& p, uint32_t d0, uint64_t a0, uint64_t b0,
                                          uint32_t a16, uint32_t b16, uint32_t m16, uint32_t idesc, uint32_t bn,
-                                         bool first, uint32_t a_tm) {
-  issue_stage<CG, KIND, NA, NK, NM, TA>(d0, a0, b0, a16, b16, m16, idesc, bn, first, a_tm, r.issue);
+                                         bool first, uint32_t a_tm, volatile int* abort_p) {
+  if constexpr (LO) {
+    issue_stage<CG, KIND, NA, NK, NM, TA, 0, 1>(d0, a0, b0, a16, b16, m16, idesc, bn, first, a_tm, r.issue);
+    if (!warp_wait(smem_u32(&r.full_lo[r.stage]), r.phase, p.wd, abort_p, SITE_GEMM_MMA)) return false;
+    tc_fence_after();
+    issue_stage<CG, KIND, NA, NK, NM, TA, 1, 3>(d0, a0, b0, a16, b16, m16, idesc, bn, first, a_tm, r.issue);
+  } else {
+    issue_stage<CG, KIND, NA, NK, NM, TA>(d0, a0, b0, a16, b16, m16, idesc, bn, first, a_tm, r.issue);
+  }
   if constexpr (CG == 1) umma_commit(smem_u32(&r.empty[r.stage]), r.issue);
   else umma_commit_pair(smem_u32(&r.empty[r.stage]), (uint16_t)3, r.issue);
   if (++r.stage == p.stages) { r.stage = 0; r.phase ^= 1u; }
+  return true;
 }
 
 // The MMA issuer's K-loop for one tile, specialised on the stage's shape
@@ -252,7 +261,7 @@ __device__ __forceinline__ void mma_step(MmaRing& r, const GemmParams& p, uint32
 // four-MMA K-steps).  Under split release (256 x 256 tiles) the first K-step
 // is peeled off; elsewhere it stays in the loop to keep the code small.
 // Returns false if a wait gave up.
-template <int CG, int KIND, int TA, int NA, int NK, int NM>
+template <int CG, int KIND, int TA, int LO, int NA, int NK, int NM>
 __device__ __forceinline__ bool mma_tile(MmaRing& r, const GemmParams& p, const Tile& T, uint32_t d0, uint32_t base,
                                          uint32_t tmem_base, uint32_t use, volatile int* abort_p) {
   constexpr int L = (KIND == 1) ? 2 : 1;
@@ -268,13 +277,17 @@ __device__ __forceinline__ bool mma_tile(MmaRing& r, const GemmParams& p, const 
       // row block 0 now, row block 1 once the epilogue has drained it from
       // the previous tile
       if (!warp_wait(smem_u32(&r.full[r.stage]), r.phase, p.wd, abort_p, SITE_GEMM_MMA)) return false;
+      if constexpr (LO)
+        if (!warp_wait(smem_u32(&r.full_lo[r.stage]), r.phase, p.wd, abort_p, SITE_GEMM_MMA)) return false;
       tc_fence_after();
       const uint64_t a0 = desc0 + (uint64_t)((uint32_t)r.stage * stage16);
       const uint64_t b0 = a0 + (uint64_t)boff16;
       issue_stage<CG, KIND, NA, NK, 1, TA>(d0, a0, b0, a16, b16, m16, T.idesc, bn, true, 0u, r.issue);
       if (!warp_wait(smem_u32(&r.acce[1]), (use & 1u) ^ 1u, p.wd, abort_p, SITE_GEMM_MMA)) return false;
       tc_fence_after();
-      mma_step<CG, KIND, NA, NK, 1, TA>(r, p, d0 + bn, a0 + (uint64_t)m16, b0, a16, b16, m16, T.idesc, bn, true, 0u);
+      if (!mma_step<CG, KIND, NA, NK, 1, TA, LO>(r, p, d0 + bn, a0 + (uint64_t)m16, b0, a16, b16, m16, T.idesc, bn,
+                                                 true, 0u, abort_p))
+        return false;
       kt0 = 1;
     }
   }
@@ -283,8 +296,9 @@ __device__ __forceinline__ bool mma_tile(MmaRing& r, const GemmParams& p, const 
     tc_fence_after();
     const uint64_t a0 = desc0 + (uint64_t)((uint32_t)r.stage * stage16);
     const uint32_t a_tm = TA ? tmem_base + (uint32_t)(p.a_col0 + r.stage * p.a_cols) : 0u;
-    mma_step<CG, KIND, NA, NK, NM, TA>(r, p, d0, a0, a0 + (uint64_t)boff16, a16, b16, m16, T.idesc, bn, kt == 0,
-                                       a_tm);
+    if (!mma_step<CG, KIND, NA, NK, NM, TA, LO>(r, p, d0, a0, a0 + (uint64_t)boff16, a16, b16, m16, T.idesc, bn,
+                                                kt == 0, a_tm, abort_p))
+      return false;
   }
   return true;
 }
@@ -303,12 +317,13 @@ __device__ __forceinline__ void stage_chunk(uint32_t sbuf, int lane, const uint3
   }
 }
 
-template <int CG, int KIND, int TA, int MAXG>
+template <int CG, int KIND, int TA, int LO, int MAXG>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     gemm_kernel(const __grid_constant__ TensorMaps maps, const __grid_constant__ GroupTableT<MAXG> g,
                 const GemmParams p) {
   extern __shared__ __align__(1024) uint8_t dsmem[];
   __shared__ __align__(8) uint64_t full_bar[kMaxStages];
+  __shared__ __align__(8) uint64_t full_lo_bar[LO ? kMaxStages : 1];
   __shared__ __align__(8) uint64_t empty_bar[kMaxStages];
   __shared__ __align__(8) uint64_t accf_bar[2];
   __shared__ __align__(8) uint64_t acce_bar[2];
@@ -332,6 +347,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) {
       mbar_init(smem_u32(&full_bar[s]), 1);
+      if constexpr (LO) mbar_init(smem_u32(&full_lo_bar[s]), 1);
       mbar_init(smem_u32(&empty_bar[s]), 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -378,29 +394,33 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         decode_tile<CG, L>(t, p, g, rank, T, qh);
         const CUtensorMap* ma = &maps.a[T.ma];
         const CUtensorMap* mb = &maps.b[T.mb];
+        const uint32_t tx = LO ? T.tx / 2u : T.tx;     // bytes a barrier of the stage counts
         for (int kt = 0; kt < p.Kt; ++kt) {
           if (!warp_wait(smem_u32(&empty_bar[stage]), phase ^ 1u, p.wd, abort_p, SITE_GEMM_PRODUCER)) {
             ok = false;
             break;
           }
-          const uint32_t fb = smem_u32(&full_bar[stage]);
-          uint32_t fbc = fb;
-          if constexpr (CG == 1) {
-            if (issue) mbar_arrive_expect_tx(fb, T.tx);
-            __syncwarp();
-          } else {
-            // The leader arms its own full barrier for both CTAs' bytes; the
-            // peer only points its TMA completions at that barrier (a
-            // completion that lands before the arming leaves the phase pending
-            // until the leader's arrival).
-            fbc = mapa_shared(fb, 0);
-            if (rank == 0 && issue) mbar_arrive_expect_tx(fb, 2u * T.tx);
-            __syncwarp();
-          }
           const uint32_t sbase = base + (uint32_t)stage * p.stage_bytes;
           const uint32_t bbase = sbase + (uint32_t)(L * p.n_atoms) * T.a_part;
+          uint32_t fb = 0, fbc = 0;
 #pragma unroll
           for (int h = 0; h < L; ++h) {
+            if (h == 0 || LO) {
+              fb = smem_u32(h == 0 ? &full_bar[stage] : &full_lo_bar[stage]);
+              if constexpr (CG == 1) {
+                if (issue) mbar_arrive_expect_tx(fb, tx);
+                __syncwarp();
+                fbc = fb;
+              } else {
+                // The leader arms its own full barrier for both CTAs' bytes; the
+                // peer only points its TMA completions at that barrier (a
+                // completion that lands before the arming leaves the phase pending
+                // until the leader's arrival).
+                fbc = mapa_shared(fb, 0);
+                if (rank == 0 && issue) mbar_arrive_expect_tx(fb, 2u * tx);
+                __syncwarp();
+              }
+            }
             for (int a = 0; a < p.n_atoms; ++a) {
               const int x = kt * p.BK + a * (p.sw / E);
               const uint32_t da = sbase + (uint32_t)(h * p.n_atoms + a) * T.a_part;
@@ -422,7 +442,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     // ------------------------------------------------------------- MMA issuer
     // the whole warp runs the loop in step; one lane issues
     if (rank == 0) {
-      MmaRing r{full_bar, empty_bar, acce_bar, 0, 0u, elect_one() ? 1u : 0u};
+      MmaRing r{full_bar, full_lo_bar, empty_bar, acce_bar, 0, 0u, elect_one() ? 1u : 0u};
       bool ok = true;
       int it = 0;
       int qh = 0;
@@ -443,14 +463,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         // the stage's MMA shape is fixed for the whole tile: dispatch once
         if (p.sw == 128) {
           if (p.n_atoms == 1)
-            ok = T.n_mblk == 1 ? mma_tile<CG, KIND, TA, 1, 4, 1>(r, p, T, d0, base, tmem_base, use, abort_p)
-                               : mma_tile<CG, KIND, TA, 1, 4, 2>(r, p, T, d0, base, tmem_base, use, abort_p);
+            ok = T.n_mblk == 1 ? mma_tile<CG, KIND, TA, LO, 1, 4, 1>(r, p, T, d0, base, tmem_base, use, abort_p)
+                               : mma_tile<CG, KIND, TA, LO, 1, 4, 2>(r, p, T, d0, base, tmem_base, use, abort_p);
           else
-            ok = T.n_mblk == 1 ? mma_tile<CG, KIND, TA, 2, 4, 1>(r, p, T, d0, base, tmem_base, use, abort_p)
-                               : mma_tile<CG, KIND, TA, 2, 4, 2>(r, p, T, d0, base, tmem_base, use, abort_p);
+            ok = T.n_mblk == 1 ? mma_tile<CG, KIND, TA, LO, 2, 4, 1>(r, p, T, d0, base, tmem_base, use, abort_p)
+                               : mma_tile<CG, KIND, TA, LO, 2, 4, 2>(r, p, T, d0, base, tmem_base, use, abort_p);
         } else {
-          ok = T.n_mblk == 1 ? mma_tile<CG, KIND, TA, 1, 2, 1>(r, p, T, d0, base, tmem_base, use, abort_p)
-                             : mma_tile<CG, KIND, TA, 1, 2, 2>(r, p, T, d0, base, tmem_base, use, abort_p);
+          ok = T.n_mblk == 1 ? mma_tile<CG, KIND, TA, LO, 1, 2, 1>(r, p, T, d0, base, tmem_base, use, abort_p)
+                             : mma_tile<CG, KIND, TA, LO, 1, 2, 2>(r, p, T, d0, base, tmem_base, use, abort_p);
         }
         if (!ok) break;
         if constexpr (CG == 1) umma_commit(smem_u32(&accf_bar[buf]), r.issue);
@@ -695,11 +715,11 @@ pm_status cached_tmap(CUtensorMap* out, const void* ptr, int dtcode, uint64_t ro
 // (programmatic dependent launch): its barriers, TMEM and tensor maps are set up
 // while that one's last blocks run.  Back to back, 1024^3 BF16 11.6-13 -> 9.1 us a launch,
 // FP32 512^3 14.7 -> 13.2, 4096 x 4096 x 256 20.7 -> 17.6, 4096^3 91.0 -> 89.2; of no account at
-// 8192^3 (now, with the roles in step, 7.0, 12.3, 16.6 and 87.7).
-template <int CG, int KIND, int TA, int MAXG>
+// 8192^3 (now, with the roles in step, 7.0, 11.2, 16.6 and 87.7).
+template <int CG, int KIND, int TA, int LO, int MAXG>
 static pm_status launch_gemm_table(const TensorMaps& maps, const GroupTableT<MAXG>& g, const GemmParams& p, int grid,
                                    size_t smem, cudaStream_t s) {
-  auto kern = gemm_kernel<CG, KIND, TA, MAXG>;
+  auto kern = gemm_kernel<CG, KIND, TA, LO, MAXG>;
   static std::once_flag once;
   static cudaError_t attr_err = cudaSuccess;
   std::call_once(once, [&] {
@@ -727,11 +747,11 @@ static pm_status launch_gemm_table(const TensorMaps& maps, const GroupTableT<MAX
 
 // One group launches with a table of one; several groups (BF16, strategy A) with
 // the whole table.
-template <int CG, int KIND, int TA>
+template <int CG, int KIND, int TA, int LO = 0>
 static pm_status launch_gemm(const TensorMaps& maps, const GroupTable& g, const GemmParams& p, int grid, size_t smem,
                              cudaStream_t s) {
   if constexpr (KIND == 0 && TA == 0) {
-    if (g.n_groups > 1) return launch_gemm_table<CG, KIND, TA, kMaxGroups>(maps, g, p, grid, smem, s);
+    if (g.n_groups > 1) return launch_gemm_table<CG, KIND, TA, LO, kMaxGroups>(maps, g, p, grid, smem, s);
   }
   GroupTableT<1> one;
   one.n_groups = 1;
@@ -744,7 +764,7 @@ static pm_status launch_gemm(const TensorMaps& maps, const GroupTable& g, const 
   one.tiles_n[0] = g.tiles_n[0];
   one.bm_idx[0] = g.bm_idx[0];
   one.bn_idx[0] = g.bn_idx[0];
-  return launch_gemm_table<CG, KIND, TA, 1>(maps, one, p, grid, smem, s);
+  return launch_gemm_table<CG, KIND, TA, LO, 1>(maps, one, p, grid, smem, s);
 }
 
 static int size_index(int v) { return v == 64 ? 0 : (v == 128 ? 1 : 2); }
@@ -896,12 +916,21 @@ static pm_status run_plan(const LaunchPlan& P, int dt, int cg, int tmem_a, cudaS
     if (dt == PM_FP32) return launch_gemm<1, 1, 1>(P.maps, P.g, P.p, P.grid, P.smem, s);
     return launch_gemm<1, 2, 1>(P.maps, P.g, P.p, P.grid, P.smem, s);
   }
+  // Low planes on a barrier of their own: rings of two stages wait for memory at
+  // every K-step, and the first pass (high planes only) then runs while the low ones
+  // arrive.  FP32 512^3 (128 x 128 x 32, 2 stages) 12.3 -> 11.2 us, 1024^3 (128 x 256 x
+  // 32, 2 stages) 30.7 -> 30.5.  Deeper rings have the stage in full before its turn
+  // and lose by the second wait (1024^3, 3 stages 17.5 -> 17.9; 64 x 64 tiles, 4 stages 20.7
+  // -> 22.0), strategy B copies both planes first (13.9 -> 14.4).
+  const bool lo = dt == PM_FP32 && P.p.stages == 2;
   if (cg == 1) {
     if (dt == PM_BF16) return launch_gemm<1, 0, 0>(P.maps, P.g, P.p, P.grid, P.smem, s);
+    if (lo) return launch_gemm<1, 1, 0, 1>(P.maps, P.g, P.p, P.grid, P.smem, s);
     if (dt == PM_FP32) return launch_gemm<1, 1, 0>(P.maps, P.g, P.p, P.grid, P.smem, s);
     return launch_gemm<1, 2, 0>(P.maps, P.g, P.p, P.grid, P.smem, s);
   }
   if (dt == PM_BF16) return launch_gemm<2, 0, 0>(P.maps, P.g, P.p, P.grid, P.smem, s);
+  if (lo) return launch_gemm<2, 1, 0, 1>(P.maps, P.g, P.p, P.grid, P.smem, s);
   if (dt == PM_FP32) return launch_gemm<2, 1, 0>(P.maps, P.g, P.p, P.grid, P.smem, s);
   return launch_gemm<2, 2, 0>(P.maps, P.g, P.p, P.grid, P.smem, s);
 }
