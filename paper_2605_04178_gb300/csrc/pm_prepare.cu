@@ -86,6 +86,16 @@ __device__ __forceinline__ void prep_store4(void* y, int64_t i, int64_t lo_off, 
   }
 }
 
+// Clears the |max| words ahead of amax_kernel.  A kernel and not a memset, so that
+// amax_kernel is set up and reads during it.  FP8 preparations in a captured graph,
+// 512^3 8.2 -> 3.9 us, 2048^3 12.3 -> 8.8, 4096^3 44.7 -> 41.0; called one by one, each
+// with its GEMM, 2048^3 22.9 -> 21.2, 4096^3 102.3 -> 101.4, below 1024^3 bound by the
+// host's calls on either side.
+__global__ void amax_clear_kernel(unsigned int* amax_bits) {
+  grid_dependents_launch();
+  if (threadIdx.x < 2) amax_bits[threadIdx.x] = 0u;
+}
+
 // Per-tensor |max| of A and B (FP8), one launch: blocks [0, a_blocks) read A,
 // the rest B, in kPrepBlock pieces with four 16-byte loads in flight per thread;
 // one atomic per block.
@@ -122,6 +132,7 @@ __global__ void __launch_bounds__(kPrepThreads) amax_kernel(const float* __restr
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < kPrepThreads / 32; ++w) m = fmaxf(m, wm[w]);
+    grid_dependency_wait();                      // after amax_clear_kernel; A and B are older than that
     atomicMax(amax_bits + (is_a ? 0 : 1), __float_as_uint(m));
   }
 }
@@ -212,9 +223,10 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const PrepArgs p) {
 
 // Launches the operand preparation of A (rows x K, or none: A == nullptr) and
 // B (K x N, or none) on stream s.  FP8: scales[2..3] collect the |max| bits
-// (zeroed by the caller before the first operand), scales[0..1] the scales.
-pm_status launch_prepare(int dt, const float* A, int64_t rows, const float* B, int K, int N, void* A_op,
-                                void* B_op, float* scales, cudaStream_t s) {
+// (cleared here if clear is set, else by the caller before the first operand),
+// scales[0..1] the scales.
+static pm_status prepare_on(int dt, const float* A, int64_t rows, const float* B, int K, int N, void* A_op, void* B_op,
+                            float* scales, bool clear, cudaStream_t s) {
   PrepArgs p = {};
   const int e = dt == PM_FP32 ? 4 : (dt == PM_BF16 ? 2 : 1);
   auto aligned = [](const void* x, int bytes) { return ((uintptr_t)x & (uintptr_t)(bytes - 1)) == 0; };
@@ -245,10 +257,23 @@ pm_status launch_prepare(int dt, const float* A, int64_t rows, const float* B, i
       ga = A ? std::max<int64_t>(1, cap * a_blocks / (a_blocks + pieces_b)) : 0;
       gb = B ? std::max<int64_t>(1, cap - ga) : 0;
     }
-    amax_kernel<<<(unsigned int)(ga + gb), kPrepThreads, 0, s>>>(A, p.nA, (unsigned int)ga, B, nB, aligned(A, 16),
-                                                                 aligned(B, 16), p.amax);
-    pm_status st = launch_status("amax_kernel");
-    if (st != PM_OK) return st;
+    if (clear) {
+      amax_clear_kernel<<<1, 32, 0, s>>>(p.amax);
+      pm_status st = launch_status("amax_clear_kernel");
+      if (st != PM_OK) return st;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned int)(ga + gb));
+    cfg.blockDim = dim3(kPrepThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = clear ? 1 : 0;                // only amax_clear_kernel may still run beside it
+    cudaError_t e1 = cudaLaunchKernelEx(&cfg, amax_kernel, A, p.nA, (unsigned int)ga, B, nB, (int)aligned(A, 16),
+                                        (int)aligned(B, 16), p.amax);
+    if (e1 != cudaSuccess) return cuda_fail(e1, "cudaLaunchKernelEx(amax_kernel)");
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)blocks);
@@ -265,6 +290,11 @@ pm_status launch_prepare(int dt, const float* A, int64_t rows, const float* B, i
   return PM_OK;
 }
 
+pm_status launch_prepare(int dt, const float* A, int64_t rows, const float* B, int K, int N, void* A_op, void* B_op,
+                         float* scales, cudaStream_t s) {
+  return prepare_on(dt, A, rows, B, K, N, A_op, B_op, scales, false, s);
+}
+
 }  // namespace pm
 
 extern "C" pm_status pm_gemm_prepare(int32_t dtype, const float* A_dev, const float* B_dev, int32_t M, int32_t N,
@@ -274,7 +304,6 @@ extern "C" pm_status pm_gemm_prepare(int32_t dtype, const float* A_dev, const fl
   PM_REQUIRE(dtype != PM_FP8E4M3 || scales_dev, PM_EINVAL, "FP8 needs scales_dev (4 floats)");
   PM_REQUIRE((K + 31) / 32 <= 65535, PM_EINVAL, "K too large for the transpose grid");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (dtype == PM_FP8E4M3) PM_CUDA(cudaMemsetAsync(scales_dev + 2, 0, 2 * sizeof(unsigned int), s));
-  return pm::launch_prepare(dtype, A_dev, M, B_dev, K, N, A_op_dev, B_op_dev, scales_dev, s);
+  return pm::prepare_on(dtype, A_dev, M, B_dev, K, N, A_op_dev, B_op_dev, scales_dev, true, s);
 }
 
