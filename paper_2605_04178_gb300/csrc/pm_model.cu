@@ -96,6 +96,9 @@ __device__ __forceinline__ float pm_exp_fast(float x) { return __expf(x); }
 __device__ __forceinline__ double pm_exp_fast(double x) { return exp(x); }
 __device__ __forceinline__ float pm_div_fast(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double pm_div_fast(double a, double b) { return a / b; }
+// a + b, not fused with the product that b may be
+__device__ __forceinline__ float pm_add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double pm_add(double a, double b) { return a + b; }
 // x / s and x / (s - 1) for a ring depth s (tabulated reciprocals for 2..7)
 template <class F>
 __device__ __forceinline__ F div_stages(F x, int s, const ThetaT<F>& th) {
@@ -228,11 +231,13 @@ __device__ __forceinline__ int64_t wave_count(int64_t tiles, int g, const ThetaT
 // W_launch > 0 overrides the working set (a grouped launch passes its own);
 // otherwise W = bytes_min of this GEMM (operands once, C once).  single >= 0
 // overrides the buffering (a grouped launch passes the launch's); otherwise
-// the tile's own.
-template <class F>
+// the tile's own.  SPACE: the launch's parameters are space_params' (measured
+// reading, L2 blend on), so the branches on them are settled when compiling:
+// 10^6 records outside the search space 16.5 -> 14.2 us, the same bits.
+template <bool SPACE = false, class F>
 __device__ __forceinline__ void gemm_forward(const pm_cfg& c, const ThetaT<F>& th, int n_sm, GemmFwdT<F>& f,
                                              F W_launch = F(-1), int single = -1) {
-  const bool measured = th.reading == PM_READING_MEASURED;
+  const bool measured = SPACE || th.reading == PM_READING_MEASURED;
   const int dt = c.dtype, g = c.cta_group;
   const F e = dt_bytes(dt), np = dt_passes(dt), l = dt_loads(dt);
   const F bytes_min = l * e * ((F)c.M * c.K + (F)c.N * c.K) + F(4) * (F)c.M * (F)c.N;
@@ -272,10 +277,10 @@ __device__ __forceinline__ void gemm_forward(const pm_cfg& c, const ThetaT<F>& t
   // hit in L2 arrive faster, Sec. III-A.2; Eq. 16's blend shape); w0 <= 0
   // switches the blend off
   f.W = W_launch > F(0) ? W_launch : bytes_min;
-  f.blend = measured && th.v[3] > F(0);
+  f.blend = SPACE || (measured && th.v[3] > F(0));
   f.E = f.blend ? pm_exp_fast(-f.W * th.inv[3]) : F(0);
   f.rho = f.blend ? F(1) + (th.v[16] - F(1)) * f.E : F(1);
-  f.T_tma = th.v[4] + (f.blend ? pm_div_fast(f.bstep * th.inv[5], f.rho) : f.bstep * th.inv[5]);   // rho = 1 unblended
+  f.T_tma = pm_add(th.v[4], f.blend ? pm_div_fast(f.bstep * th.inv[5], f.rho) : f.bstep * th.inv[5]);   // rho = 1 unblended
   const F T_sync = F(2) * th.v[12];
   // 1 - alpha = clamp(c_alpha / s, 0, 1) (literal) or clamp(c_alpha / (s - 1),
   // 0, 1) (measured: s - 1 loads in flight while one stage is consumed; a
@@ -298,7 +303,7 @@ __device__ __forceinline__ void gemm_forward(const pm_cfg& c, const ThetaT<F>& t
   f.launch = measured ? th.v[0] + th.v[13] : th.v[0];
   f.T_stage = f.launch + f.waves * (f.Kt * f.T_step + f.T_store);
   const F flops = np * F(2) * (F)c.M * (F)c.N * (F)c.K;
-  f.A_rl = th.nc_nsm == n_sm ? flops * (f.invR * f.invS) * th.inv_nsm : flops * (f.invR * f.invS) / (F)n_sm;
+  f.A_rl = SPACE || th.nc_nsm == n_sm ? flops * (f.invR * f.invS) * th.inv_nsm : flops * (f.invR * f.invS) / (F)n_sm;
   f.B_rl = bytes_min * th.inv[2];
   f.T_rl = f.launch + (f.A_rl >= f.B_rl ? f.A_rl : f.B_rl);
   f.T = f.T_stage >= f.T_rl ? f.T_stage : f.T_rl;
@@ -385,14 +390,17 @@ __device__ __forceinline__ void gemm_adjoint(const pm_cfg& c, const ThetaT<F>& t
 }
 
 // The records that the search space and the calibration table are made of take
-// a shorter way to the same values: GEMM records under the measured reading with BM, BN in {64, 128, 256}, BK in {32, 64, 128}, 2..6 stages
-// and extents below 2^20, whose counts fit in 32 bits and whose extents are
+// a shorter way to the same values: GEMM records under the measured reading with
+// BM, BN in {64, 128, 256}, BK in {32, 64, 128}, 2..6 stages and M N below 2^41,
+// whose counts fit in 32 bits (at most 2^29 + 2^26 tiles) and whose extents are
 // divided by shifts.  What depends on (dtype, cta_group) or on the stages alone
 // is looked up in shared memory: kernel parameters indexed by a lane's own value
 // are read once per distinct value.  The floating-point operations are
 // gemm_forward's, in its order, so the results are the same bits.  Both TMEM
 // strategies take it: rows of strategy B scattered over a table (the calibration's)
 // would send nearly every warp both ways (10^6 mixed records: 19.6 us, now 9.6).
+// So would extents: half of 10^6 records with M above 2^21 cost 12.9 us the
+// general way alone, 19.8 with the limit at 2^20 per extent, 8.8 here.
 struct SpaceTables {
   float4 rate[6];       // by 2 dtype + (cta_group - 1): 1 / (R S), l e, n_p, 1 / R
   uint4 conc[2];        // by cta_group - 1: the wave division d - 1, m, s1, s2
@@ -400,8 +408,15 @@ struct SpaceTables {
   float inv_s2sm[2];    // by cta_group - 1: 1 / S
 };
 
-// Whether the launch's parameters allow the short way (uniform over the launch).
-__device__ __forceinline__ bool space_tables(const Theta& th, int n_sm, SpaceTables& t) {
+// Whether a launch's parameters allow the short way.  Launches that they do not (the
+// literal reading, no L2 blend, one SM) have kernels without it: 10^6 records under the
+// literal reading 10.8 us, 11.7 in a kernel with both ways.
+template <class F>
+inline bool space_params(const ThetaT<F>& th, int n_sm) {
+  return th.reading == PM_READING_MEASURED && th.nc_nsm == n_sm && th.v[3] > F(0);
+}
+
+__device__ __forceinline__ void space_tables(const Theta& th, SpaceTables& t) {
   if (threadIdx.x < 6) {
     const int dt = threadIdx.x >> 1, g = 1 + (threadIdx.x & 1);
     const float invR = th.inv[dt_rate(dt)], invS = g == 1 ? 1.f : th.inv[14];
@@ -417,16 +432,37 @@ __device__ __forceinline__ bool space_tables(const Theta& th, int n_sm, SpaceTab
                              r > 0.f && r < 1.f ? 1.f : 0.f);
   }
   __syncthreads();
-  return th.reading == PM_READING_MEASURED && th.nc_nsm == n_sm && th.v[3] > 0.f;
 }
 
+// All conditions without a branch: the fields of a record share words, what may not
+// be set in any of them is collected in one (with early exits 10^6 records take 9.0
+// us instead of 8.75).
 __device__ __forceinline__ bool in_space(const pm_cfg& c) {
-  const unsigned tile = (unsigned)(uint16_t)c.BM | (unsigned)(uint16_t)c.BN << 16, bk = (unsigned)(uint16_t)c.BK;
-  // one bit of 64..256 in each half of `tile`, one of 32..128 in bk
-  return c.kind == PM_KIND_GEMM && (unsigned)c.tmem_a <= 1u && (unsigned)(c.stages - 2) <= 4u &&
-         (unsigned)(c.cta_group - 1) <= 1u && (unsigned)c.dtype <= 2u && (tile & ~0x01C001C0u) == 0u &&
-         (tile & 0xFFFFu) != 0u && (tile >> 16) != 0u && (tile & (tile - 0x00010001u)) == 0u && (bk & ~0xE0u) == 0u &&
-         bk != 0u && (bk & (bk - 1u)) == 0u && ((unsigned)(c.M - 1) | (unsigned)(c.N - 1) | (unsigned)(c.K - 1)) < (1u << 20);
+  const unsigned tile = (unsigned)(uint16_t)c.BM | (unsigned)(uint16_t)c.BN << 16;
+  const unsigned step = (unsigned)(uint16_t)c.BK | (unsigned)(uint8_t)c.stages << 16 | (unsigned)(uint8_t)c.cta_group << 24;
+  const unsigned type = (unsigned)(uint8_t)c.dtype | (unsigned)(uint8_t)c.kind << 8 | (unsigned)(uint8_t)c.tmem_a << 16;
+  const unsigned sign = (unsigned)(c.M - 1) | (unsigned)(c.N - 1) | (unsigned)(c.K - 1);
+  // 64..256 in each half of tile, 32..128 in BK, 0..7 stages, 0..3 groups and types,
+  // kind 0 and tmem_a 0 or 1, extents of at least 1, M N < 2^41
+  const unsigned stray = (tile & ~0x01C001C0u) | (step & 0xFCF8FF1Fu) | (type & 0x00FEFFFCu) | (sign >> 31) |
+                         (__umulhi((unsigned)c.M, (unsigned)c.N) >> 9);
+  // then one bit in each of BM, BN and BK, 2..6 stages, groups 1 and 2, types 0..2
+  const unsigned pairs = (tile & (tile - 0x00010001u)) | (step & (step - 1u) & 0xE0u);
+  return (stray | pairs) == 0u && (tile & 0xFFFFu) != 0u && (tile >> 16) != 0u && (step & 0xE0u) != 0u &&
+         ((0x7Cu >> ((step >> 16) & 7u)) & (6u >> (step >> 24)) & (7u >> (type & 3u)) & 1u) != 0u;
+}
+
+// The FP64 way keeps K exact in FP32 (small_f64) and the bytes of the operands below
+// 2^51 (large_f64).
+__device__ __forceinline__ bool in_space_f64(const pm_cfg& c) {
+  return in_space(c) && (unsigned)(c.K - 1) < (1u << 24) &&
+         ((uint64_t)((unsigned)c.M + (unsigned)c.N) * (unsigned)c.K) >> 48 == 0ull;
+}
+
+// Lanes of the warp that have a record in this turn of a loop over records; i is this lane's.
+__device__ __forceinline__ unsigned lanes_with_record(int64_t i, int64_t n) {
+  const int64_t left = n - (i - (threadIdx.x & 31));
+  return left >= 32 ? 0xffffffffu : (1u << (int)left) - 1u;
 }
 
 // The whole numbers of a record of the space: tensor-pipe instructions of a
@@ -466,12 +502,12 @@ __device__ __forceinline__ void gemm_forward_space(const pm_cfg& c, const Theta&
   f.invR = rt.w;
   f.invS = tab.inv_s2sm[gi];
   const int kb = BK >> 6;                                        // 32, 64, 128 -> 0, 1, 2
-  const unsigned tm = (unsigned)(c.M + (BM << gi) - 1) >> (6 + (BM >> 7) + gi);
-  const unsigned tn = (unsigned)(c.N + BN - 1) >> (6 + (BN >> 7));
+  const unsigned tm = ((unsigned)c.M + (unsigned)((BM << gi) - 1)) >> (6 + (BM >> 7) + gi);
+  const unsigned tn = ((unsigned)c.N + (unsigned)(BN - 1)) >> (6 + (BN >> 7));
   const unsigned x = ((tm * tn) << gi) + nc.x;
   const unsigned q = __umulhi(nc.y, x);
   f.waves = (float)(int)((q + ((x - q) >> nc.z)) >> nc.w);
-  f.Kt = (float)(int)((unsigned)(c.K + BK - 1) >> (5 + kb));
+  f.Kt = (float)(int)(((unsigned)c.K + (unsigned)(BK - 1)) >> (5 + kb));
   f.D = (float)(4 * BM * BN);
   const SpaceInts si = space_ints(c);
   f.n_instr = (float)si.n_instr;
@@ -486,7 +522,7 @@ __device__ __forceinline__ void gemm_forward_space(const pm_cfg& c, const Theta&
   f.blend = true;
   f.E = pm_exp_fast(-f.W * th.inv[3]);
   f.rho = 1.f + (th.v[16] - 1.f) * f.E;
-  f.T_tma = __fadd_rn(th.v[4], pm_div_fast(f.bstep * th.inv[5], f.rho));   // not fused with the quotient
+  f.T_tma = pm_add(th.v[4], pm_div_fast(f.bstep * th.inv[5], f.rho));
   const float T_sync = 2.f * th.v[12];
   f.oma = dp.x;
   f.inv_s = dp.y;
@@ -524,10 +560,9 @@ struct SpaceHost<double> {
   double oma[8], inv_s[8], inv_s1[8];        // by stages: 1 - alpha, 1 / s, and 1 / (s - 1) where alpha is free, else 0
   double rho_m1, c3, ni10, ni11, t_sync, launch;   // rho_L2 - 1, its share of w0's slope, -1/BW^2, 2 L_mbar, launch
   uint4 conc[2];                             // as SpaceTables
-  int ok;                                    // the launch's parameters allow the short way
 };
 
-static SpaceHost<double> make_space(const ThetaT<double>& th, int n_sm) {
+static SpaceHost<double> make_space(const ThetaT<double>& th) {
   SpaceHost<double> k = {};
   for (int i = 0; i < 6; ++i) {
     k.inv_r[i] = th.inv[6 + i / 2];
@@ -548,10 +583,9 @@ static SpaceHost<double> make_space(const ThetaT<double>& th, int n_sm) {
   k.launch = th.v[0] + th.v[13];
   for (int i = 0; i < 2; ++i)
     k.conc[i] = make_uint4(th.nc[i].d - 1u, th.nc[i].m, (unsigned)th.nc[i].s1, (unsigned)th.nc[i].s2);
-  k.ok = th.reading == PM_READING_MEASURED && th.nc_nsm == n_sm && th.v[3] > 0.0;
   return k;
 }
-static SpaceHost<float> make_space(const ThetaT<float>&, int) { return {}; }
+static SpaceHost<float> make_space(const ThetaT<float>&) { return {}; }
 
 // A positive integer that FP32 holds exactly, through FP32's bits.
 __device__ __forceinline__ double small_f64(int v) {
@@ -570,9 +604,9 @@ __device__ __forceinline__ double space_row(const pm_cfg& c, const ThetaT<double
   const int passes = dt == PM_FP32 ? 3 : 1, le = dt == PM_FP32 ? 8 : 2 >> (dt - 1);
   const SpaceInts si = space_ints(c);
   const long long mn = (long long)c.M * c.N;
-  const double W = large_f64(le * ((long long)(c.M + c.N) * c.K) + 4 * mn);
-  const unsigned tm = (unsigned)(c.M + (BM << gi) - 1) >> (6 + (BM >> 7) + gi);
-  const unsigned tn = (unsigned)(c.N + BN - 1) >> (6 + (BN >> 7));
+  const double W = large_f64(le * (((long long)c.M + c.N) * c.K) + 4 * mn);
+  const unsigned tm = ((unsigned)c.M + (unsigned)((BM << gi) - 1)) >> (6 + (BM >> 7) + gi);
+  const unsigned tn = ((unsigned)c.N + (unsigned)(BN - 1)) >> (6 + (BN >> 7));
   const uint4 nc = k.conc[gi];
   const unsigned x = ((tm * tn) << gi) + nc.x, q = __umulhi(nc.y, x);
   const double waves = large_f64((long long)((q + ((x - q) >> nc.z)) >> nc.w));
@@ -777,14 +811,19 @@ __device__ __forceinline__ pm_cfg load_cfg(const pm_cfg* p) {
 // 10^7 114 -> 69 us with the short way of gemm_forward_space.  Six blocks per SM
 // (40 registers, no spills): 48 warps hide the latency of the dependent FP32
 // chain better than 40 or, at 32 registers, 64 (10^6: 11.0 us).
+// SPACE: the launch's parameters allow the short way.  Its records do not choose
+// together: a vote of the warp costs 0.4 us per 10^6 records, and only tables that
+// mix tiles inside and outside the search space pay for both ways (every other
+// record outside: 18.7 us, 14.1 by the general way alone).
+template <bool SPACE>
 __global__ void __launch_bounds__(256, 6) model_predict_kernel(const pm_cfg* __restrict__ cfgs, int64_t n, Theta th,
                                                             int n_sm, float* __restrict__ out) {
   __shared__ SpaceTables tab;
-  const bool space = space_tables(th, n_sm, tab);
+  if constexpr (SPACE) space_tables(th, tab);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const pm_cfg c = load_cfg(cfgs + i);
     float t;
-    if (space && in_space(c)) {
+    if (SPACE && in_space(c)) {
       GemmFwd f;
       gemm_forward_space(c, th, tab, f);
       t = f.T;
@@ -792,7 +831,7 @@ __global__ void __launch_bounds__(256, 6) model_predict_kernel(const pm_cfg* __r
       t = __int_as_float(0x7fc00000);
     } else if (c.kind == PM_KIND_GEMM) {
       GemmFwd f;
-      gemm_forward(c, th, n_sm, f);
+      gemm_forward<SPACE>(c, th, n_sm, f);
       t = f.T;
     } else {
       ProbeFwd f;
@@ -862,7 +901,11 @@ constexpr int grad_min_blocks() { return sizeof(F) == 4 ? 4 : 2; }
 // over a cluster of CL blocks: partials[j * records + r] is component j of
 // record r.  CL > 1 for few records, so that they use CL times as many SMs;
 // the sums are the same, term by term, whatever CL.
-template <class F, int CL>
+//
+// SPACE as in model_predict_kernel.  In FP64 the GEMM records of a warp go one way
+// together: one outside the space takes the others with it (every other of 10^6
+// records outside: 616 -> 437 us; 495 by the general way alone).
+template <class F, int CL, bool SPACE>
 __global__ void __launch_bounds__(kGradThreads / CL, CL == 1 ? grad_min_blocks<F>() : 1)
     model_grad_kernel(const pm_cfg* __restrict__ cfgs, int64_t n, const __grid_constant__ ThetaT<F> th,
                       const __grid_constant__ SpaceHost<F> sh, int n_sm, const F* __restrict__ t_meas,
@@ -873,14 +916,13 @@ __global__ void __launch_bounds__(kGradThreads / CL, CL == 1 ? grad_min_blocks<F
   const int records = (int)(gridDim.x / CL), rec = (int)(blockIdx.x / CL), part = (int)(blockIdx.x % CL);
   // the short way's tables, in shared memory (lanes index them by their own record)
   __shared__ std::conditional_t<sizeof(F) == 4, SpaceTables, SpaceHost<F>> tab;
-  bool space;
-  if constexpr (sizeof(F) == 4) {
-    space = space_tables(th, n_sm, tab);
+  if constexpr (!SPACE) {
+  } else if constexpr (sizeof(F) == 4) {
+    space_tables(th, tab);
   } else {
     const int* from = reinterpret_cast<const int*>(&sh);
     for (int w = threadIdx.x; w < (int)(sizeof(sh) / 4); w += kThreads) reinterpret_cast<int*>(&tab)[w] = from[w];
     __syncthreads();
-    space = sh.ok != 0;
   }
   F acc[NREC];                                   // loss, then the gradient
 #pragma unroll
@@ -893,7 +935,14 @@ __global__ void __launch_bounds__(kGradThreads / CL, CL == 1 ? grad_min_blocks<F
 #pragma unroll
     for (int j = 0; j < NP; ++j) d[j] = F(0);
     F T;
-    if (space && in_space(c)) {
+    bool space = false;
+    if constexpr (SPACE && sizeof(F) == 4) space = in_space(c);
+    if constexpr (SPACE && sizeof(F) == 8) {
+      space = in_space_f64(c);
+      const bool outside = __any_sync(lanes_with_record(i, n), !space && c.kind == PM_KIND_GEMM);
+      space = space && !outside;
+    }
+    if (space) {
       if constexpr (sizeof(F) == 4) {
         GemmFwd f;
         gemm_forward_space(c, th, tab, f);
@@ -906,7 +955,7 @@ __global__ void __launch_bounds__(kGradThreads / CL, CL == 1 ? grad_min_blocks<F
       T = (F)__int_as_float(0x7fc00000);
     } else if (c.kind == PM_KIND_GEMM) {
       GemmFwdT<F> f;
-      gemm_forward(c, th, n_sm, f);
+      gemm_forward<SPACE>(c, th, n_sm, f);
       T = f.T;
       gemm_adjoint(c, th, f, F(1), d);
     } else if constexpr (sizeof(F) == 4) {
@@ -1572,14 +1621,16 @@ extern "C" pm_status pm_model_predict(const pm_cfg* cfgs_dev, int64_t n, const p
   PM_REQUIRE(cfgs_dev && theta_host && t_out_dev && n_sm > 0, PM_EINVAL, "null pointer or n_sm <= 0");
   PM_REQUIRE(((uintptr_t)cfgs_dev & 7) == 0, PM_EINVAL, "cfgs_dev must be 8-byte aligned");
   const int64_t want = (n + 255) / 256;
-  // one resident wave that walks the records up to eight rounds (10^6 records 8.9 us,
-  // 9.6 with 16 blocks per SM); past that smaller shares even out the SMs' speeds
-  // (10^7: 72 against 66 us)
+  const Theta th = to_theta(theta_host, n_sm);
+  const bool space = space_params(th, n_sm);
+  // with the short way one resident wave that walks the records up to eight rounds (10^6
+  // records 8.9 us, 9.6 with 16 blocks per SM); past that, and without it at every
+  // size, smaller shares even out the SMs' speeds (10^7: 72 against 66 us)
   const int64_t resident = (int64_t)std::max(1, sm_count()) * 6;
-  const int64_t cap = want <= 8 * resident ? resident : (int64_t)std::max(1, sm_count()) * 16;
+  const int64_t cap = space && want <= 8 * resident ? resident : (int64_t)std::max(1, sm_count()) * 16;
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, cap));
-  model_predict_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(cfgs_dev, n, to_theta(theta_host, n_sm),
-                                                                            n_sm, t_out_dev);
+  auto kern = space ? model_predict_kernel<true> : model_predict_kernel<false>;
+  kern<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(cfgs_dev, n, th, n_sm, t_out_dev);
   return launch_status("model_predict_kernel");
 }
 
@@ -1600,7 +1651,8 @@ static pm_status launch_grad(const pm_cfg* cfgs, int64_t n, const ThetaT<F>& th,
   // fit at once).  The
   // FP32 kernel is bound by one thread's latency and gains nothing.
   constexpr int CL = sizeof(F) == 8 ? 8 : 1;
-  const SpaceHost<F> sh = make_space(th, n_sm);
+  const bool space = space_params(th, n_sm);
+  const SpaceHost<F> sh = space ? make_space(th) : SpaceHost<F>{};
   cudaLaunchConfig_t cfg = {};
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -1613,10 +1665,12 @@ static pm_status launch_grad(const pm_cfg* cfgs, int64_t n, const ThetaT<F>& th,
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, model_grad_kernel<F, CL>, cfgs, n, th, sh, n_sm, t_meas, partials);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, space ? model_grad_kernel<F, CL, true> : model_grad_kernel<F, CL, false>,
+                                       cfgs, n, th, sh, n_sm, t_meas, partials);
     if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchKernelEx(model_grad_kernel)");
   } else {
-    model_grad_kernel<F, 1><<<records, kGradThreads, 0, s>>>(cfgs, n, th, sh, n_sm, t_meas, partials);
+    auto kern = space ? model_grad_kernel<F, 1, true> : model_grad_kernel<F, 1, false>;
+    kern<<<records, kGradThreads, 0, s>>>(cfgs, n, th, sh, n_sm, t_meas, partials);
     pm_status st = launch_status("model_grad_kernel");
     if (st != PM_OK) return st;
   }
