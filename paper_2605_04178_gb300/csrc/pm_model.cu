@@ -1267,7 +1267,7 @@ template <class F>
 struct Schedule {
   F tau[kMaxGroups];
   int64_t per[kMaxGroups + 1];
-  int rem[kMaxGroups + 1];
+  unsigned rem[kMaxGroups + 1];          // below P < 2^32
   int16_t list[kMaxGroups], pos[kMaxGroups];
   uint8_t key[kMaxGroups];               // class << 5 | rank inside its 32 groups
   int cls[kGroupClasses][32];            // groups per class and 32 groups, then their first positions
@@ -1366,7 +1366,7 @@ __device__ void grouped_list(const int16_t* bm, const int16_t* bn, const int64_t
     const int64_t off = sc.per[i + 1] + sc.part[i >> 5];
     const int64_t per = P > 0 ? off / P : 0;      // no worker: the caller rejects the launch
     sc.per[i + 1] = per;
-    sc.rem[i + 1] = (int)(off - per * P);
+    sc.rem[i + 1] = (unsigned)(off - per * P);
   }
   if (threadIdx.x == 0) { sc.per[0] = 0; sc.rem[0] = 0; }
   __syncthreads();
