@@ -379,7 +379,7 @@ pm_status pm_autotune_pick(const int32_t* MNK_dev, int64_t n, int32_t dtype, con
  * measured reading).  Host arrays of G entries (G <= 1024); *t_pred_host in
  * seconds, NaN for a cta_group 2 launch when n_sm < 2.  The grouped model calls
  * keep one 87 KB block of page-locked host memory per calling thread, until the
- * thread ends or calls pm_shutdown.  Synchronises. */
+ * thread ends or any thread calls pm_shutdown.  Synchronises. */
 pm_status pm_grouped_predict(int32_t G, const int32_t* M_host, int32_t N, int32_t K, const int16_t* BM_host,
                              const int16_t* BN_host, int32_t BK, int32_t stages, int32_t cta_group, int32_t dtype,
                              const pm_params* theta_host, int32_t n_sm, float* t_pred_host, void* stream);
@@ -479,11 +479,12 @@ pm_status pm_segment_predict(const pm_segment* segs_dev, int64_t n, const pm_par
 const char* pm_last_error(void);
 
 /* Releases what the library holds beyond its static device arrays: its pool
- * of concurrent-probe streams on every device, and the calling thread's
- * host-transfer pipeline (streams, events), page-locked block of the grouped
- * model calls and TMA descriptor caches; it also
- * forgets the cached device addresses of the static arrays (the watchdog
- * word, the allocation-free gradient's scratch) and the cached SM counts.
+ * of concurrent-probe streams on every device, the page-locked blocks of the
+ * grouped model calls of every thread (it waits for such calls in progress),
+ * and the calling thread's host-transfer pipeline (streams, events) and TMA
+ * descriptor caches; it also forgets the cached device addresses of the
+ * static arrays (the watchdog word, the allocation-free gradient's scratch)
+ * and the cached SM counts.
  * Call it before a device reset (cudaDeviceReset reloads the module, so a
  * cached address would go stale).  Work already queued on those streams
  * completes.  Any later call re-creates or looks up what it needs.  Always

@@ -1780,25 +1780,52 @@ namespace pm {
 // thread: the kernels read the row counts and tiles from it and write their
 // results to it, so a call is one launch and one wait.  Device scratch from the
 // stream's pool and four copies cost about 270 us a call (the pool gives its
-// memory back at every wait and maps it again).  A call waits for its kernel
-// before it returns, so the block is never in use by two calls; it is given
-// back when the thread ends and by pm_shutdown.
+// memory back at every wait and maps it again).  A call holds its thread's block
+// until it has waited for its kernel and copied the results.  The blocks of all
+// threads are in one list, so that pm_shutdown gives every one of them back: a
+// device reset frees them, whichever thread prepares it.  A thread's block is
+// also given back when the thread ends.
 constexpr size_t kGroupScratch = 4 * kMaxGroups + 2 * 2 * 20 * kMaxGroups + 512;
 
+struct GroupScratch;
+static std::mutex g_group_list_mu;
+static GroupScratch* g_group_list = nullptr;
+
 struct GroupScratch {
+  std::mutex mu;                         // held by the thread's call, and to release the block
   char* p = nullptr;
+  GroupScratch *prev = nullptr, *next = nullptr;
+  GroupScratch() {
+    std::lock_guard<std::mutex> lk(g_group_list_mu);
+    next = g_group_list;
+    if (next) next->prev = this;
+    g_group_list = this;
+  }
+  ~GroupScratch() {
+    {
+      std::lock_guard<std::mutex> lk(g_group_list_mu);
+      if (next) next->prev = prev;
+      (prev ? prev->next : g_group_list) = next;
+    }
+    release();
+  }
   void release() {
+    std::lock_guard<std::mutex> lk(mu);
     if (p) cudaFreeHost(p);
     p = nullptr;
   }
-  ~GroupScratch() { release(); }
 };
 static thread_local GroupScratch g_group_scratch;
 
-void release_group_scratch_this_thread() { g_group_scratch.release(); }
+void release_group_scratch() {
+  std::lock_guard<std::mutex> lk(g_group_list_mu);
+  for (GroupScratch* g = g_group_list; g; g = g->next) g->release();
+}
 
-static pm_status group_scratch(char** out) {
+// The calling thread's block, held by `hold` until it goes out of scope.
+static pm_status group_scratch(char** out, std::unique_lock<std::mutex>& hold) {
   GroupScratch& g = g_group_scratch;
+  hold = std::unique_lock<std::mutex>(g.mu);
   if (!g.p) {
     void* p = nullptr;
     PM_CUDA(cudaHostAlloc(&p, kGroupScratch, cudaHostAllocPortable | cudaHostAllocMapped));
@@ -1818,7 +1845,8 @@ static pm_status grouped_candidates(int32_t G, const int32_t* M_host, int32_t N,
   PM_REQUIRE(N > 0 && K > 0 && dtype >= 0 && dtype <= 2, PM_EINVAL, "bad N, K or dtype");
   for (int q = 0; q < G; ++q) PM_REQUIRE(M_host[q] > 0, PM_EINVAL, "M[%d] <= 0", q);
   char* buf = nullptr;
-  pm_status st = group_scratch(&buf);
+  std::unique_lock<std::mutex> hold;
+  pm_status st = group_scratch(&buf, hold);
   if (st != PM_OK) return st;
   float* pt = reinterpret_cast<float*>(buf);                    // 20 floats
   int32_t* pM = reinterpret_cast<int32_t*>(buf + 128);          // G
@@ -1864,7 +1892,8 @@ static pm_status grouped_eval(int32_t G, const int32_t* M_host, int32_t N, int32
   }
   const int n_out = grad ? 1 + NP : 1;
   char* buf = nullptr;
-  pm_status st = group_scratch(&buf);
+  std::unique_lock<std::mutex> hold;
+  pm_status st = group_scratch(&buf, hold);
   if (st != PM_OK) return st;
   F* pt = reinterpret_cast<F*>(buf);                            // 1 + NP values
   int32_t* pM = reinterpret_cast<int32_t*>(buf + 256);          // G each

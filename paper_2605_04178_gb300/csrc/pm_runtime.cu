@@ -54,8 +54,8 @@ unsigned int* watchdog_word() {
 
 // The allocation-free gradient's scratch address cache (pm_model.cu).
 void clear_grad_scratch_cache();
-// The calling thread's page-locked block of the grouped model calls (pm_model.cu).
-void release_group_scratch_this_thread();
+// The page-locked blocks of the grouped model calls, of every thread (pm_model.cu).
+void release_group_scratch();
 
 // Forget the per-device addresses of the library's static device arrays and
 // the cached SM counts; the next call looks them up again.  A device reset
@@ -279,7 +279,7 @@ extern "C" pm_status pm_clock_sample(pm_clock* out) {
 extern "C" pm_status pm_shutdown(void) {
   pm::release_stream_pool();
   pm::release_host_pipe_this_thread();
-  pm::release_group_scratch_this_thread();
+  pm::release_group_scratch();
   pm::clear_tmap_caches_this_thread();
   pm::clear_device_address_caches();
   pm::clear_grad_scratch_cache();
