@@ -40,6 +40,7 @@
 #include <mutex>
 #include <vector>
 
+#include "pm_footprint.cuh"
 #include "pm_internal.cuh"
 
 namespace pm {
@@ -727,7 +728,7 @@ static pm_status launch_gemm_table(const TensorMaps& maps, const GroupTableT<MAX
   static std::once_flag once;
   static cudaError_t attr_err = cudaSuccess;
   std::call_once(once, [&] {
-    attr_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - 1024);
+    attr_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemDynamic);
   });
   if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute(gemm_kernel)");
   cudaLaunchConfig_t cfg = {};
@@ -818,8 +819,6 @@ static pm_status plan_launch(int dt, int cg, int BK, int stages, int tmem_a, int
   p.lo_row_b = L == 2 ? (int)b_rows : 0;
   g.n_groups = G;
   g.tile_off[0] = 0;
-  int acc = 0, max_mblk = 1;
-  uint32_t stage = 0;
   bool used_m[3] = {false, false, false}, used_n[3] = {false, false, false};
   // rows of each problem in the stacked A and C (the caller's order), then
   // the table's order: largest tile (BM x BN) first, ties in the caller's
@@ -846,38 +845,29 @@ static pm_status plan_launch(int dt, int cg, int BK, int stages, int tmem_a, int
     g.bm_idx[i] = (uint8_t)size_index(bm);
     g.bn_idx[i] = (uint8_t)size_index(bn);
     used_m[g.bm_idx[i]] = used_n[g.bn_idx[i]] = true;
-    const int n_mblk = (bm + 127) / 128;
-    acc = std::max(acc, (bm < 128 && cg == 2) ? bn / 2 : n_mblk * bn);
-    max_mblk = std::max(max_mblk, n_mblk);
-    stage = std::max(stage, (uint32_t)(L * p.n_atoms) * (uint32_t)(bm + bn / cg) * (uint32_t)p.sw);
   }
-  p.acc_cols = acc;
-  // strategy B: one 8-column slot per 128-row x 32-byte A slice, per stage
-  p.a_cols = tmem_a ? L * (BK * e / 4) * max_mblk : 0;
-  const int a_ring = stages * p.a_cols;
-  p.nbuf = (2 * acc + a_ring <= 512) ? 2 : 1;
+  const GemmFootprint fp = gemm_footprint(e, L, cg, BK, stages, tmem_a, G, BMv, BNv);
+  p.acc_cols = fp.acc_cols;
+  p.a_cols = fp.a_cols;
+  p.nbuf = fp.nbuf;
   // split release when one buffer of two 128-row blocks holds the whole tile
   // (every group: BM = 256 per CTA) and nothing else lives in TMEM
   bool all_two_blocks = true;
   for (int q = 0; q < G; ++q) all_two_blocks = all_two_blocks && BMv[q] == 256;
   p.split = (p.nbuf == 1 && all_two_blocks && tmem_a == 0) ? 1 : 0;
-  p.a_col0 = p.nbuf * acc;
-  int cols = 32;
-  while (cols < p.nbuf * acc + a_ring) cols <<= 1;
-  p.alloc_cols = cols;
-  p.stage_bytes = stage;
-  P.smem = (size_t)stages * stage + 1024;
+  p.a_col0 = p.nbuf * p.acc_cols;
+  p.alloc_cols = fp.alloc_cols;
+  p.stage_bytes = fp.stage_bytes;
+  P.smem = fp.smem;
   // epilogue staging after the ring: two 4 KB buffers per warp (which TMA stores
   // need), or one where no more fits (256 x 64 x 64 BF16, 5 stages, 8000 x 8000 x 512:
   // 152 -> 124 us, now 115; with 7999 columns 465 -> 139, now 105); without any, lanes store their rows
-  p.staging_off = (uint32_t)stages * stage;
+  p.staging_off = (uint32_t)stages * fp.stage_bytes;
+  p.staged = fp.staged;
   p.tma_store = 0;
   p.c_rows = (int)sum_m;
   const bool c_ok = (N % 4) == 0 && ((uintptr_t)C & 15) == 0;
   p.vec = c_ok ? 1 : 0;
-  const size_t room = (size_t)(232448 - 1024) - P.smem;
-  p.staged = room >= 32768 ? 2 : (room >= 16384 ? 1 : 0);
-  P.smem += (size_t)p.staged * 16384;
   if (c_ok && p.staged == 2) {
     pm_status st = cached_tmap(&P.maps.c, C, TMAP_F32, (uint64_t)sum_m, (uint64_t)N, 32u, 32u, 128);
     if (st != PM_OK) return st;

@@ -6,6 +6,7 @@
 #include <mutex>
 #include <vector>
 
+#include "pm_footprint.cuh"
 #include "pm_internal.cuh"
 
 namespace pm {
@@ -528,7 +529,9 @@ static pm_status probe_launch(const pm_probe_args* a, void* buf0, void* buf1, vo
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(grid);
       cfg.blockDim = dim3(128);
-      cfg.dynamicSmemBytes = 49 * 1024;
+      // a pair holds its share of shared memory for its 256 columns (pm_footprint.cuh)
+      const size_t smem = cg == 2 ? pair_smem(49 * 1024, 256) : 49 * 1024;
+      cfg.dynamicSmemBytes = smem;
       cfg.stream = s;
       cudaLaunchAttribute attr[1];
       attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -540,7 +543,7 @@ static pm_status probe_launch(const pm_probe_args* a, void* buf0, void* buf1, vo
       cudaError_t e;
 #define PM_MMA_PROBE(CG, KIND)                                                                           \
   do {                                                                                                   \
-    cudaFuncSetAttribute(mma_probe_kernel<CG, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, 49 * 1024); \
+    cudaFuncSetAttribute(mma_probe_kernel<CG, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
     e = cudaLaunchKernelEx(&cfg, mma_probe_kernel<CG, KIND>, a->n, M, N, out, wd);                     \
   } while (0)
       if (cg == 1) {
