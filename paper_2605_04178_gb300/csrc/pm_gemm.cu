@@ -488,7 +488,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     // --------------------------------------------------------------- epilogue
     const int q = warp & 3;                               // TMEM lane quarter of this warp
     float scale = 1.f;
-    if constexpr (KIND == 2) scale = 1.f / (__ldg(p.scales) * __ldg(p.scales + 1));
+    if constexpr (KIND == 2) scale = 1.f / (p.scales[0] * p.scales[1]);
     const bool vec = p.vec != 0;
     const uint32_t stage_base = base + p.staging_off;     // the epilogue warps' staging buffers
     uint32_t sb = 0;

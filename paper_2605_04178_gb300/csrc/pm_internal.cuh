@@ -224,7 +224,10 @@ __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
 // up while the previous kernel of its stream still runs, once every block of that
 // kernel has called grid_dependents_launch (or has ended).  grid_dependency_wait
 // returns when the previous kernel has ended and its writes are visible; a kernel
-// launched without the attribute passes at once.
+// launched without the attribute passes at once.  What that kernel may have written
+// is read after the wait, by plain loads: __ldg and const __restrict__ promise data
+// that does not change while this kernel runs, which here begins before the other
+// ends, and they let the compiler move a load ahead of the wait.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

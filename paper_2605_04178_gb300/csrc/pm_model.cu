@@ -1006,8 +1006,8 @@ __global__ void __launch_bounds__(kGradThreads / CL, CL == 1 ? grad_min_blocks<F
 // records on 152 SMs), takes 3.7 us where one block with strided records took
 // 8.5, and it is set up while the partial sums are made (programmatic launch:
 // 1.2 to 2.5 us less from one call to the next).
-__global__ void __launch_bounds__(32) model_grad_finish_kernel(const double* __restrict__ partials, int records,
-                                                               int64_t n, double* __restrict__ out) {
+__global__ void __launch_bounds__(32) model_grad_finish_kernel(const double* partials, int records, int64_t n,
+                                                               double* out) {
   constexpr int kBatch = 20;
   grid_dependency_wait();                        // the records are complete and visible
   const double* p = partials + (int64_t)blockIdx.x * records;

@@ -137,7 +137,8 @@ __global__ void __launch_bounds__(kPrepThreads) amax_kernel(const float* __restr
   }
 }
 
-// Vector accesses are used where the pointers and the row lengths allow them
+// Plain loads: A and B may be the results of the kernel that this one overlaps
+// (grid_dependency_wait).  Vector accesses are used where the pointers and the row lengths allow them
 // (a_vec, b_vec_in, b_vec_out: four elements of the type, checked on the
 // host); otherwise, and in partial blocks, one element at a time.  A 64 x 64
 // tile of B goes through shared memory with rows of 65 words: four k of one
@@ -164,13 +165,22 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const PrepArgs p) {
       const float4* x = reinterpret_cast<const float4*>(p.A + base) + tid;
       float4 v[kPrepVec];
 #pragma unroll
-      for (int u = 0; u < kPrepVec; ++u) v[u] = __ldg(x + u * kPrepThreads);
+      for (int u = 0; u < kPrepVec; ++u) v[u] = x[u * kPrepThreads];
 #pragma unroll
       for (int u = 0; u < kPrepVec; ++u)
         prep_store4<MODE>(p.A_op, base + 4 * (tid + u * kPrepThreads), p.nA, v[u], s);
     } else {
-      const int64_t end = min(base + (int64_t)kPrepBlock, p.nA);
-      for (int64_t i = base + tid; i < end; i += kPrepThreads) prep_store1<MODE>(p.A_op, i, p.nA, __ldg(p.A + i), s);
+      // eight loads ahead of their stores (for all the compiler knows the stores go to where the loads read)
+      const float* x = p.A + base;
+      const int left = (int)min((int64_t)kPrepBlock, p.nA - base);
+      for (int j0 = tid; j0 < left; j0 += 8 * kPrepThreads) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = j0 + u * kPrepThreads < left ? x[j0 + u * kPrepThreads] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (j0 + u * kPrepThreads < left) prep_store1<MODE>(p.A_op, base + j0 + u * kPrepThreads, p.nA, v[u], s);
+      }
     }
     return;
   }
@@ -182,7 +192,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const PrepArgs p) {
     float4 v[kPrepVec];
 #pragma unroll
     for (int u = 0; u < kPrepVec; ++u)
-      v[u] = __ldg(reinterpret_cast<const float4*>(p.B + (size_t)(k0 + r0 + 16 * u) * p.N + n0 + c));
+      v[u] = *reinterpret_cast<const float4*>(p.B + (size_t)(k0 + r0 + 16 * u) * p.N + n0 + c);
 #pragma unroll
     for (int u = 0; u < kPrepVec; ++u) {
       float* t = tile + (r0 + 16 * u) * S + c;
@@ -195,7 +205,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const PrepArgs p) {
 #pragma unroll
     for (int u = 0; u < kPrepTile / 4; ++u) {
       const int k = k0 + r0 + 4 * u;
-      v[u] = (in && k < p.K) ? __ldg(p.B + (size_t)k * p.N + n0 + c) : 0.f;
+      v[u] = (in && k < p.K) ? p.B[(size_t)k * p.N + n0 + c] : 0.f;
     }
 #pragma unroll
     for (int u = 0; u < kPrepTile / 4; ++u) tile[(r0 + 4 * u) * S + c] = v[u];
