@@ -235,8 +235,8 @@ pm_status pm_probe_run(const pm_probe_args* args, void* buf0, void* buf1, void* 
  * [N,K] (K-major, FP32: hi then lo), `scales_dev` 4 floats. */
 pm_status pm_gemm_operand_bytes(int32_t dtype, int32_t M, int32_t N, int32_t K, size_t* a_bytes, size_t* b_bytes);
 
-/* Operand preparation (async): casts row-major FP32 A [M,K] and B [K,N]
- * into the tensor-core operand formats.  BF16: round to nearest even.
+/* Operand preparation (async, K at most 2,097,120): casts row-major FP32
+ * A [M,K] and B [K,N] into the tensor-core operand formats.  BF16: round to nearest even.
  * FP8 e4m3: per-tensor scale s = 448/max|X| (FP32 division), codes
  * RNE-saturated from s*X; scales_dev[0] = s_A, scales_dev[1] = s_B.
  * FP32: hi = tf32_rn(X), lo = tf32_rn(X - hi).  scales_dev (4 floats) is

@@ -19,9 +19,9 @@
 // Two TMEM accumulator buffers when they fit, so the epilogue of tile i
 // overlaps the main loop of tile i+1.  When one accumulator fills TMEM (two
 // 128-row blocks of 256 columns) the two row blocks are released separately:
-// tile i+1 starts on row block 0 while the epilogue still drains row block 1.  Each CTA of a pair loads its own A
-// rows and half of B (traffic 2 M_A + M_B per pair, no multicast); the pair
-// leader issues the cta_group::2 MMAs.
+// tile i+1 starts on row block 0 while the epilogue still drains row block 1.
+// Each CTA of a pair loads its own A rows and half of B (traffic 2 M_A + M_B per
+// pair, no multicast); the pair leader issues the cta_group::2 MMAs.
 //
 // Warps 0 and 1 run their K-loops converged (waits, addresses and descriptors
 // in all lanes) and one elected lane issues, each instruction under its
@@ -549,13 +549,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             // two buffers: through the warp's staging buffer, so that the lanes
             // write along the rows of C, one 128-byte row segment per store (four
             // where rows are 16-byte multiples) instead of one element of 32
-            // rows, which cost 32 requests a store and bound the kernel.  BF16
-            // 4096 x 4095 x 256 96 -> 30 us (22.5 with the roles in step), 4096 x 4095 x
-            // 4096 181 -> 117 (106), 1000 x 1003 x 1040 17.9 -> 11.2 (9.1), FP8 300 x 2941
-            // x 528 14.5 -> 8.2 (7.1).  (Chunks whose rows
-            // allow 16-byte stores are left to the lanes beside TMA and in 64-row
-            // tiles: staging them made the single-buffered 256 x 256 tiles of grouped
-            // launches 2-3 % slower.)
+            // rows, which costs 32 requests a store and bounded the kernel (BF16 4096 x
+            // 4095 x 256 96 -> 30 us, 1000 x 1003 x 1040 17.9 -> 11.2, FP8 300 x 2941 x 528
+            // 14.5 -> 8.2).  Chunks whose rows allow 16-byte stores are left to the lanes
+            // beside TMA and in 64-row tiles: staging them made the single-buffered 256 x
+            // 256 tiles of grouped launches 2-3 % slower.
             const uint32_t sbuf = stage_base + (uint32_t)((p.staged * q + (sb & 1)) * 4096);
             if (lane == 0) bulk_wait_read<1>();          // the buffer's previous TMA store has read it
             __syncwarp();
@@ -635,9 +633,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     tc_fence_after();
     tmem_dealloc<CG>(tmem_base, (uint32_t)p.alloc_cols);
   } else if (warp > 1 && lane == 0) {
-    // staged stores complete before exit, beside the release of TMEM: 0.15-0.2 us of
-    // a launch (1024^3 BF16 6.9 -> 6.7, FP32 512^3 11.2 -> 11.05) against a wait ahead of
-    // the barrier
+    // staged stores complete before exit, beside the release of TMEM: 0.15 us of a
+    // launch against a wait ahead of the barrier (1024^3 BF16 6.45 -> 6.3)
     bulk_wait_all();
   }
 }
@@ -718,9 +715,9 @@ pm_status cached_tmap(CUtensorMap* out, const void* ptr, int dtcode, uint64_t ro
 
 // The kernel is launched to overlap the end of the previous kernel of its stream
 // (programmatic dependent launch): its barriers, TMEM and tensor maps are set up
-// while that one's last blocks run.  Back to back, 1024^3 BF16 11.6-13 -> 9.1 us a launch,
-// FP32 512^3 14.7 -> 13.2, 4096 x 4096 x 256 20.7 -> 17.6, 4096^3 91.0 -> 89.2; of no account at
-// 8192^3 (now, with the roles in step, 7.0, 11.2, 16.6 and 87.7).
+// while that one's last blocks run.  Back to back in a graph, without it and with it:
+// 1024^3 BF16 6.8 / 6.3 us a launch, 1000 x 1003 x 1040 10.0 / 8.6, FP8 300 x 2941 x 528
+// 7.4 / 6.3; of no account at 8192^3.
 template <int CG, int KIND, int TA, int LO, int MAXG>
 static pm_status launch_gemm_table(const TensorMaps& maps, const GroupTableT<MAXG>& g, const GemmParams& p, int grid,
                                    size_t smem, cudaStream_t s) {
@@ -860,8 +857,8 @@ static pm_status plan_launch(int dt, int cg, int BK, int stages, int tmem_a, int
   p.stage_bytes = fp.stage_bytes;
   P.smem = fp.smem;
   // epilogue staging after the ring: two 4 KB buffers per warp (which TMA stores
-  // need), or one where no more fits (256 x 64 x 64 BF16, 5 stages, 8000 x 8000 x 512:
-  // 152 -> 124 us, now 115; with 7999 columns 465 -> 139, now 105); without any, lanes store their rows
+  // need), or one where no more fits (256 x 64 x 64 BF16, 5 stages, 8000 x 8000 x 512
+  // without it 130 us, with it 98; with 7999 columns 424 and 99); without any, lanes store their rows
   p.staging_off = (uint32_t)stages * fp.stage_bytes;
   p.staged = fp.staged;
   p.tma_store = 0;
@@ -1092,10 +1089,12 @@ extern "C" pm_status pm_gemm_autotune(const pm_cfg* shape, int32_t k, const pm_p
 // Two staging buffers per chunked operand; events order reuse.  The chunks of
 // either buffer have their own compute stream: a chunk's product has few tiles
 // and is bound by its K-loop's latency (44 us for 512 x 4096 x 4096, on 32 SMs),
-// so one after another they, not the host link, set the pace.  BF16 4096^3 in 8 / 16 /
-// 32 chunks 907 / 1250 / 1950 -> 890 / 1036 / 1448 us (floor 640: both inputs over the
-// link), FP32 1024^3 in 4 / 8 chunks 170 / 266 -> 125 / 178.  At 8 chunks the result's
-// way back beside the inputs (155 against 195 GB/s alone) is the longest chain.
+// so with many chunks they, one after another, and not the host link set the pace.
+// On one compute stream and on two: BF16 4096^3 in 8 / 16 / 32 chunks 880 / 1179 / 1887
+// and 876 / 1029 / 1421 us (floor 640: both inputs over the link), FP32 1024^3 in 4 / 8
+// chunks 145 / 249 and 118 / 174.  Up to 8 chunks of 4096^3, and at 8192^3, the second
+// stream gains nothing: the result's way back beside the inputs (155 against 195 GB/s
+// alone) is the longest chain.
 namespace pm {
 
 struct HostPipe {
@@ -1201,7 +1200,7 @@ extern "C" pm_status pm_gemm_host(const pm_cfg* cfg, const float* A_host, const 
   float* b32 = reinterpret_cast<float*>(ws + Lh.off_b32);
   void* bop = ws + Lh.off_bop;
   float* scales = reinterpret_cast<float*>(ws + Lh.off_scales);
-  PM_REQUIRE((K + 31) / 32 <= 65535, PM_EINVAL, "K too large for the transpose grid");
+  PM_REQUIRE(K <= kPrepareMaxK, PM_EINVAL, "K %d is above %d", K, kPrepareMaxK);
   PM_CUDA(cudaEventRecord(P.start, caller));
   PM_CUDA(cudaStreamWaitEvent(P.s_in, P.start, 0));
   for (cudaStream_t sc : P.s_comp) PM_CUDA(cudaStreamWaitEvent(sc, P.start, 0));

@@ -24,6 +24,8 @@ unsigned int* watchdog_word();
 unsigned long long watchdog_limit_ns();
 // Number of SMs of the current device.
 int sm_count();
+// Largest K of a preparation: the limit that callers know, kept as it is.
+constexpr int kPrepareMaxK = 65535 * 32;
 // Operand preparation on stream s (pm_prepare.cu): A (rows x K, nullptr: none) and B (K x N, nullptr: none).
 pm_status launch_prepare(int dt, const float* A, int64_t rows, const float* B, int K, int N, void* A_op, void* B_op,
                          float* scales, cudaStream_t s);

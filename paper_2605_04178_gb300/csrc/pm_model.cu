@@ -3,10 +3,11 @@
 // calibration (Sec. III-D), and the model-driven autotuner (Sec. III-B
 // adaptive tile selection, Sec. VI autotuning guidance).
 //
-// One thread per configuration, FP32 arithmetic, integer tile counts.  The
-// explicit-configuration kernels stream 24-byte records (HBM-bound at
-// 24-28 B per configuration); the autotuner decodes the configuration from
-// the thread index and reads nothing per configuration (ALU-bound).
+// FP32 arithmetic (FP64 for the fit), integer tile counts.  The kernels over
+// explicit configurations take a 24-byte record per thread; the autotuner tabulates
+// the terms of its tiles or decodes a tile from the thread index, and reads a shape
+// for 180 of them.  All of them are bound by ALU issue (FP64: by its units), not by
+// memory.
 #include <math.h>
 
 #include <algorithm>
@@ -398,7 +399,7 @@ __device__ __forceinline__ void gemm_adjoint(const pm_cfg& c, const ThetaT<F>& t
 // are read once per distinct value.  The floating-point operations are
 // gemm_forward's, in its order, so the results are the same bits.  Both TMEM
 // strategies take it: rows of strategy B scattered over a table (the calibration's)
-// would send nearly every warp both ways (10^6 mixed records: 19.6 us, now 9.6).
+// would send nearly every warp both ways (10^6 mixed records 19.6 us, 9.7 this way).
 // So would extents: half of 10^6 records with M above 2^21 cost 12.9 us the
 // general way alone, 19.8 with the limit at 2^20 per extent, 8.8 here.
 struct SpaceTables {
@@ -806,9 +807,9 @@ __device__ __forceinline__ pm_cfg load_cfg(const pm_cfg* p) {
   return c;
 }
 
-// Bound: ALU issue (about 215 warp-instructions per 32 configurations in the search
-// space, 377 for any others; 28 bytes each).  10^6 configurations 13.2 -> 8.9 us,
-// 10^7 114 -> 69 us with the short way of gemm_forward_space.  Six blocks per SM
+// Bound: ALU issue (some 215 warp-instructions per 32 configurations in the search
+// space, 377 by the general way; 28 bytes each).  10^6 configurations 12.9 -> 8.8 us,
+// 10^7 114 -> 70 us with the short way of gemm_forward_space.  Six blocks per SM
 // (40 registers, no spills): 48 warps hide the latency of the dependent FP32
 // chain better than 40 or, at 32 registers, 64 (10^6: 11.0 us).
 // SPACE: the launch's parameters allow the short way.  Its records do not choose
@@ -892,10 +893,10 @@ __device__ __forceinline__ T warp_sum_each(T (&v)[N], int& index) {
 template <class F>
 constexpr int grad_min_blocks() { return sizeof(F) == 4 ? 4 : 2; }
 
-// Bound: FP32 ALU issue (10^6 configurations 25.1 -> 22.2 us with the sums by
-// halving, 15.3 us with the short way of gemm_forward_space; 10^7 218 -> 133 us);
-// FP64 at every size the FP64 units (1,901 configurations 26.8 -> 12.8 us on
-// clusters, 10.3 with space_row; 10^6 486 -> 312 us).
+// Bound: FP32 ALU issue, FP64 at every size the FP64 units.  With the sums by halving,
+// the short way and, in FP64, the clusters and space_row, against one general way with
+// a tree per sum; both launches of a call: FP32 10^6 configurations 33.5 -> 18.2 us, 10^7
+// 224 -> 131; FP64 1,901 configurations 31.6 -> 13.8, 10^6 494 -> 320.
 //
 // One partial record per kGradThreads threads, the threads of a record spread
 // over a cluster of CL blocks: partials[j * records + r] is component j of
@@ -1041,9 +1042,9 @@ static int grad_blocks(int64_t n) {
 // warp takes a shape: its lanes work out the shape's terms (bytes, rho, the
 // roofline bounds, one wave count per cta_group, BM and BN) and evaluate up to
 // six tiles each from the table with the arithmetic of gemm_forward.  Bound:
-// ALU issue; BF16 (121 valid tiles), best tile of 5,556 shapes 17.1 -> 7.0 us and
-// of 555,555 shapes 1385 -> 352 us against a whole model evaluation per
-// (shape, tile); best eight of 5,556 shapes 47.1 -> 14.0 us.
+// ALU issue; BF16 (121 valid tiles), best tile of 5,556 shapes 17.1 -> 7.3 us and
+// of 555,555 shapes 1383 -> 359 us against a whole model evaluation per
+// (shape, tile); best eight of 5,556 shapes 46.9 -> 14.3 us.
 //
 // autotune_shape_kernel (few shapes): a block per shape, thread t evaluates
 // tile t.  Bound: latency; it has no table to build before the first shape, so
@@ -1624,8 +1625,8 @@ extern "C" pm_status pm_model_predict(const pm_cfg* cfgs_dev, int64_t n, const p
   const Theta th = to_theta(theta_host, n_sm);
   const bool space = space_params(th, n_sm);
   // with the short way one resident wave that walks the records up to eight rounds (10^6
-  // records 8.9 us, 9.6 with 16 blocks per SM); past that, and without it at every
-  // size, smaller shares even out the SMs' speeds (10^7: 72 against 66 us)
+  // records 8.8 us, 9.9 with 16 blocks per SM); past that, and without it at every
+  // size, smaller shares even out the SMs' speeds (10^7: 78.5 us in one wave, 70.2)
   const int64_t resident = (int64_t)std::max(1, sm_count()) * 6;
   const int64_t cap = space && want <= 8 * resident ? resident : (int64_t)std::max(1, sm_count()) * 16;
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, cap));
@@ -1645,11 +1646,10 @@ namespace pm {
 template <class F>
 static pm_status launch_grad(const pm_cfg* cfgs, int64_t n, const ThetaT<F>& th, int n_sm, const F* t_meas,
                              double* partials, int records, double* out, cudaStream_t s) {
-  // FP64, few records: a cluster of eight one-warp blocks per record.  Measured
-  // with / without clusters, before space_row: 1,901 configurations 12.8 / 21.0 us,
-  // 20,000 15.9 / 21.3, 30,000 19.6 / 21.4, 38,000 33.2 / 21.5 (the clusters no longer
-  // fit at once).  The
-  // FP32 kernel is bound by one thread's latency and gains nothing.
+  // FP64, few records: a cluster of eight one-warp blocks per record.  Both launches of
+  // a call with / without clusters: 1,901 configurations 13.8 / 18.8 us, 20,000 16.2 /
+  // 19.0, 25,856 17.5 / 19.1, 30,000 the same, 38,000 28.8 / 19.5 (the clusters no longer fit
+  // at once).  The FP32 kernel is bound by one thread's latency and gains nothing.
   constexpr int CL = sizeof(F) == 8 ? 8 : 1;
   const bool space = space_params(th, n_sm);
   const SpaceHost<F> sh = space ? make_space(th) : SpaceHost<F>{};

@@ -5,13 +5,13 @@
 // needs the maximum first).  Both operands go through one launch, so a small
 // product pays one launch instead of two, and every thread has four 16-byte
 // loads in flight and writes four elements at a time.  Measured for A and B
-// together, events around the call, against one element per thread and store
+// together, calls in a row in a graph, against one element per thread and store
 // in a launch per operand:
-//   BF16  8192^3   261 -> 124 us (6.49 TB/s)    4096^3   80 ->  40 us
-//   FP32  8192^3   374 -> 252 us (6.38 TB/s)    4096^3  106 ->  71 us
-//   FP8   8192^3   407 -> 185 us                4096^3  127 ->  55 us
-//   BF16  8192 x 8191 x 4096 (N odd)  141 -> 71 us
-// FP8 at 8192^3 is the time of two reads and one write at the copy rate.
+//   BF16  8192^3   246 -> 112 us (7.2 TB/s)    4096^3   67 ->  29 us
+//   FP32  8192^3   358 -> 237 us (6.8 TB/s)    4096^3   92 ->  59 us
+//   FP8   8192^3   390 -> 173 us               4096^3  113 ->  41 us
+//   BF16  8192 x 8191 x 4096 (N odd)  127 -> 58 us
+// FP8 at 8192^3 is the time of two reads and one write at 7 TB/s.
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 
@@ -150,8 +150,8 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const PrepArgs p) {
   const int tid = threadIdx.x;
   grid_dependents_launch();                      // a GEMM on these operands may be set up
   grid_dependency_wait();                        // what the previous kernel of the stream wrote or still read is settled
-  // FP8: the amax pass read A then B front to back; walking the blocks from
-  // the end finds the part of the matrices that is still in L2
+  // FP8: the maximum pass read A and B at once, each front to back; walking the
+  // blocks from the end starts with what it read last of B, which is still in L2
   const unsigned int blk = MODE == PM_FP8E4M3 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
   float s = 1.f;
   if constexpr (MODE == PM_FP8E4M3) {
@@ -312,7 +312,7 @@ extern "C" pm_status pm_gemm_prepare(int32_t dtype, const float* A_dev, const fl
   PM_REQUIRE(dtype >= 0 && dtype <= 2 && M > 0 && N > 0 && K > 0, PM_EINVAL, "bad dtype or shape");
   PM_REQUIRE(A_dev && B_dev && A_op_dev && B_op_dev, PM_EINVAL, "null pointer");
   PM_REQUIRE(dtype != PM_FP8E4M3 || scales_dev, PM_EINVAL, "FP8 needs scales_dev (4 floats)");
-  PM_REQUIRE((K + 31) / 32 <= 65535, PM_EINVAL, "K too large for the transpose grid");
+  PM_REQUIRE(K <= pm::kPrepareMaxK, PM_EINVAL, "K %d is above %d", K, pm::kPrepareMaxK);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   return pm::prepare_on(dtype, A_dev, M, B_dev, K, N, A_op_dev, B_op_dev, scales_dev, true, s);
 }
