@@ -201,6 +201,8 @@ def _stream(stream):
 def params(theta) -> pm_params:
     th = np.ascontiguousarray(theta, dtype=np.float32)
     assert th.size == N_PARAMS, "theta has %d entries, not %d" % (th.size, N_PARAMS)
+    if th.ndim != 1:
+        raise TypeError("theta is not a vector: shape %s" % (th.shape,))
     return pm_params.from_buffer_copy(th)
 
 
